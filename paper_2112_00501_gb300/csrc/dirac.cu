@@ -10,6 +10,7 @@
 //    over blockIdx.y.
 //  - k_clover_apply: out = C psi or C^-1 psi.
 #include "hop.cuh"
+#include "fix64.cuh"
 #include "hop16.cuh"
 #include "mgc_host.h"
 
@@ -185,6 +186,136 @@ int launch_gauge_pack(const Geom &g, const double *canon_dev, int prec, int comp
     return MGC_OK;
 }
 
+// ------------------------------------------------------------------ fixed-point operands
+// q = x 2^s (|q| < 2^62) as limbs, the low one never -2^31 so that it can be negated
+__device__ __forceinline__ int2 fix_store(fix_t q)
+{
+    int hi, lo;
+    fix_limbs(q, hi, lo);
+    return make_int2(hi, max(lo, -0x7fffffff));
+}
+
+// The links in units of 2^-60; *bad is set unless the rows and columns of every
+// link have norm 1 to 1e-3, which bounds the operator's sums.
+__global__ void k_fix_links(Geom g, Gauge64 U, int4 *__restrict__ out, int *bad)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= g.V) return;
+    const int mu = blockIdx.y;
+    Cx<double> u[9];
+    U.load(i, mu, u);
+    int4 *o = out + (((size_t)(i >> g.lvb) * 4 + mu) * 9 << g.lvb) + (i & ((1 << g.lvb) - 1));
+    bool fine = true;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const double row = norm2(u[3 * a]) + norm2(u[3 * a + 1]) + norm2(u[3 * a + 2]);
+        const double col = norm2(u[a]) + norm2(u[3 + a]) + norm2(u[6 + a]);
+        fine = fine && fabs(row - 1.0) < 1e-3 && fabs(col - 1.0) < 1e-3;
+    }
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        const int2 r = fix_store(__double2ll_rn(u[k].r * 0x1p60)), m = fix_store(__double2ll_rn(u[k].i * 0x1p60));
+        o[(size_t)k << g.lvb] = make_int4(r.x, r.y, m.x, m.y);
+    }
+    if (!fine) atomicOr(bad, 1);
+}
+
+// C/kappa in units of 2^(e - 58) with the site's exponent e, |C/kappa| < 2^e.
+// The quotient is formed with its remainder, so the 58 bits are C's own.
+__global__ void k_fix_clover(Geom g, Clover64 C, double kappa, int4 *__restrict__ out, int *__restrict__ ex, int *bad)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= g.V) return;
+    const double2 *q = C.p + ((size_t)(i >> g.lvb) * 36 << g.lvb) + (i & ((1 << g.lvb) - 1));
+    double m = 0;
+    bool fine = true;
+    for (int k = 0; k < 36; ++k) {
+        const double2 v = q[(size_t)k << g.lvb];
+        m = fmax(m, fmax(fabs(v.x), fabs(v.y)));
+        fine = fine && isfinite(v.x) && isfinite(v.y);
+    }
+    const int e = ilogb(m / kappa) + 2;  // one to spare for the quotient's rounding
+    if (!fine || m == 0 || e < -16 || e > 16) {
+        atomicOr(bad, 1);
+        return;
+    }
+    ex[i] = e;
+    const double s = ldexp(1.0, 58 - e);
+    int4 *o = out + ((size_t)(i >> g.lvb) * 36 << g.lvb) + (i & ((1 << g.lvb) - 1));
+    auto one = [&](double c) {
+        const double hi = c / kappa, lo = fma(-hi, kappa, c) / kappa;
+        const fix_t t = __double2ll_rn(hi * s);
+        return fix_store(t + __double2ll_rn((hi * s - (double)t) + lo * s));
+    };
+    for (int k = 0; k < 36; ++k) {
+        const double2 v = q[(size_t)k << g.lvb];
+        const int2 a = one(v.x), b = one(v.y);
+        o[(size_t)k << g.lvb] = make_int4(a.x, a.y, b.x, b.y);
+    }
+}
+
+int launch_fix_links(const Geom &g, const double2 *U64, int4 *out, int *d_bad, cudaStream_t s)
+{
+    k_fix_links<<<dim3(grid_for(g.V, 128), 4), 128, 0, s>>>(g, Gauge64{(double2 *)U64, g.lvb}, out, d_bad);
+    MGC_CUDA(cudaGetLastError());
+    count(1, (double)g.V * (2 * 576.0));
+    return MGC_OK;
+}
+
+int launch_fix_clover(const Geom &g, const double2 *C64, double kappa, int4 *out, int *ex, int *d_bad, cudaStream_t s)
+{
+    k_fix_clover<<<grid_for(g.V, 128), 128, 0, s>>>(g, Clover64{(double2 *)C64, g.lvb}, kappa, out, ex, d_bad);
+    MGC_CUDA(cudaGetLastError());
+    count(1, (double)g.V * (2 * 576.0 + 4.0));
+    return MGC_OK;
+}
+
+// D, D^dagger at FP64 in block fixed point (fix64.cuh).  24^3 x 48: 383 us
+// against 1259 us with FP64 instructions (2.7 TB/s of compulsory bytes against
+// 0.8); the FMA pipe's heavy half, where the widening products run, is busy 67 %
+// of the time.  Four blocks per SM (128 registers) and three (168) measure the
+// same; five spill (429 us).
+template <bool DAG, int LVB>
+__global__ void __launch_bounds__(FIX_THREADS, 4)
+    k_dirac_fix(Geom g, Spinor64 in, Spinor64 out, FixLinks U, FixClover C, Gauge64 Ud, Clover64 Cd, double kappa)
+{
+    __shared__ int4 slots[(FIX_SPINOR_SLOTS + FIX_LINK_SLOTS) * FIX_THREADS];
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= g.V) return;
+    const int r = blockIdx.y;
+    Spinor64 src = shift_rhs(in, r, g.V), dst = shift_rhs(out, r, g.V);
+    if (LVB > 0) {
+        g.lvb = LVB;
+#pragma unroll
+        for (int mu = 0; mu < 4; ++mu) g.lb[mu] = LVB / 4;
+        src.lvb = dst.lvb = U.lvb = C.lvb = LVB;
+    }
+    if (!fix_dirac_site<DAG>(g, i, src, dst, U, C, kappa, slots + threadIdx.x)) fix_fallback<DAG>(g, i, src, dst, Ud, Cd, kappa);
+}
+
+template <int LVB>
+static void dirac_fix_launch(const mgc_clover_s *op, bool dag, Spinor64 in, Spinor64 out, int nrhs, cudaStream_t s)
+{
+    const mgc_gauge_s *ga = op->gauge;
+    const Geom &g = ga->lat->g;
+    const FixLinks U{ga->UQ, g.lvb};
+    const FixClover C{op->CQ, op->CE, g.lvb};
+    const Gauge64 Ud{ga->U64, g.lvb};
+    const Clover64 Cd{op->C64, g.lvb};
+    dim3 grid(grid_for(g.V, FIX_THREADS), nrhs);
+    if (dag) k_dirac_fix<true, LVB><<<grid, FIX_THREADS, 0, s>>>(g, in, out, U, C, Ud, Cd, op->kappa);
+    else k_dirac_fix<false, LVB><<<grid, FIX_THREADS, 0, s>>>(g, in, out, U, C, Ud, Cd, op->kappa);
+}
+
+static void dirac_fix_dispatch(const mgc_clover_s *op, bool dag, Spinor64 in, Spinor64 out, int nrhs, cudaStream_t s)
+{
+    const Geom &g = op->gauge->lat->g;
+    const bool cube = g.lb[0] == g.lb[1] && g.lb[1] == g.lb[2] && g.lb[2] == g.lb[3];
+    if (cube && g.lvb == 8) dirac_fix_launch<8>(op, dag, in, out, nrhs, s);
+    else if (cube && g.lvb == 4) dirac_fix_launch<4>(op, dag, in, out, nrhs, s);
+    else dirac_fix_launch<0>(op, dag, in, out, nrhs, s);
+}
+
 // ------------------------------------------------------------------ D, D^dagger
 // LVB > 0: cubic domains of 2^LVB sites, whose extents the compiler then knows
 // (shifts and masks of the index arithmetic become constants); LVB == 0: any
@@ -318,7 +449,9 @@ int launch_dirac(const mgc_clover_s *op, int prec, bool dag, const void *in, voi
     const mgc_gauge_s *ga = op->gauge;
     const Geom &g = ga->lat->g;
     if (!has_prec(ga, prec)) return fail(MGC_ERR_INVALID_ARG, "no copy of the operator at this precision");
-    if (prec == 64) {
+    if (prec == 64 && op->CQ) {
+        dirac_fix_dispatch(op, dag, sp64(g, in), sp64(g, out), nrhs, s);
+    } else if (prec == 64) {
         dirac_dispatch(g, dag, sp64(g, in), sp64(g, out), Gauge64{ga->U64, g.lvb}, Clover64{op->C64, g.lvb},
                        op->kappa, nrhs, s);
     } else if (prec == 32) {

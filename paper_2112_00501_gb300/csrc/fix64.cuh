@@ -1,0 +1,493 @@
+// The FP64 operator in block fixed point: products of 62-bit fixed-point
+// numbers on the integer multiply-add units.
+//
+// GB300 issues 2 FP64 fused multiply-adds per clock and SM, but 32 widening
+// integer multiply-adds (32 x 32 + 64 bits; the first measured with eight
+// independent chains per thread, the second from the busy cycles of the pipe).  A product of two-limb integers
+// a = a1 2^32 + a0 whose low limbs are balanced (|a0| <= 2^31, random sign)
+// needs three of them, hh += a1 b1 and mid += a1 b0 + a0 b1: the dropped a0 b0
+// is below the last bit kept.  A multiply-add of more precision than FP64's
+// therefore takes three instructions of 1/16 the cost, which turns the operator
+// from one bound by the FP64 pipe into one bound by instruction issue and HBM.
+//
+// Scales.  Links are u = q 2^-60 (unitary to 1e-3, so |q| <= 2^60).  The clover
+// term is stored divided by kappa, q = (C/kappa) 2^(58 - e_C), e_C the site's
+// exponent (|C/kappa| < 2^e_C), so that D psi = kappa (C/kappa psi - H psi) needs
+// one multiplication per component.  A thread adds its eight hops and the
+// clover term in 64-bit integers in units of 2^(E - 56), E at least the
+// exponent of the largest component of psi at the nine sites: a neighbour's
+// components are brought to that unit as they are read (Q = psi 2^(60 - E)),
+// and where a neighbour exceeds E the sum is shifted down.  Sum bounds: a hop's
+// row has |sum| <= 4.9 (unitary rows, |h| <= 2 2^E), eight of them 2^5.3, the
+// clover term 2^5.46 (E >= e_psi + e_C - 2), together below 2^62.5 units; the
+// middle sums stay below 2^62.8 (two-norm bound for the links, eleven terms of
+// 2^57 + 2^59 for the clover).
+//
+// A site is computed with FP64 instructions instead (fix_fallback) when its own
+// or a neighbour's components span more than 2^27, include some but not only
+// zeros, are not finite, or lie outside 2^-894 .. 2^961: wide-range and sparse
+// fields keep the FP64 operator's component-wise accuracy, infinities and NaN
+// propagate, and no conversion needs a test of its own.  Gaussian components
+// fall below 2^-27 of their neighbourhood's largest once in 10^8.
+//
+// Error against 64 bits: each hop truncates at 2^(E - 56) (the -1/2 mean is
+// added back once), against FP64's rounding of every partial sum at 2^(E - 53).
+#pragma once
+
+#include "hop.cuh"
+#include "tma.cuh"
+
+namespace mgc {
+
+typedef long long fix_t;
+
+constexpr int FIX_EMIN = 0x80;   // smallest biased exponent the fixed-point path takes
+constexpr int FIX_EMAX = 0x7c0;  // first biased exponent it does not
+
+// threads of a block, and the 16-byte staging slots each has in shared memory
+// (slot k of thread t at [k][t]): a neighbour's spinor and a link
+constexpr int FIX_THREADS = 128;
+constexpr int FIX_SPINOR_SLOTS = 12, FIX_LINK_SLOTS = 9;
+
+// 16-byte asynchronous copies global -> shared, read back by the thread that
+// issued them, so no barrier is involved
+__device__ __forceinline__ void fix_copy16(int4 *dst, const void *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void fix_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void fix_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// links: the plane order of Gauge64, a complex entry as (re hi, re lo, im hi, im lo)
+struct FixLinks {
+    const int4 *p;
+    int lvb;
+    __device__ __forceinline__ const int4 *at(int i, int mu) const
+    {
+        return p + (((size_t)(i >> lvb) * 4 + mu) * 9 << lvb) + (i & ((1 << lvb) - 1));
+    }
+};
+
+// C/kappa: the plane order of Clover64, and the exponent of every site
+struct FixClover {
+    const int4 *p;
+    const int *e;
+    int lvb;
+    __device__ __forceinline__ const int4 *at(int i) const
+    {
+        return p + ((size_t)(i >> lvb) * 36 << lvb) + (i & ((1 << lvb) - 1));
+    }
+};
+
+__device__ __forceinline__ fix_t mac64(int a, int b, fix_t c) { return c + (fix_t)a * (fix_t)b; }
+__device__ __forceinline__ fix_t mul64(int a, int b) { return (fix_t)a * (fix_t)b; }
+// -x (and the limbs below) as 32-bit numbers of unknown origin: where the compiler
+// can see them it sign-extends first and multiplies 64-bit numbers (850 of the
+// 2,640 products a site, each in four instructions).  The products themselves
+// stay in C: as mad.wide in inline PTX a third came out as a multiplication and
+// a separate 64-bit addition.
+__device__ __forceinline__ int fix_neg(int x)
+{
+    int r;
+    asm("neg.s32 %0, %1;" : "=r"(r) : "r"(x));
+    return r;
+}
+
+// largest and smallest magnitude of three words read as FP32 bit patterns: the
+// high words of doubles order like the doubles; NaN patterns (exponents from
+// 0x7f8 on) stay NaN in the maximum
+__device__ __forceinline__ float max3abs(float a, float b, float c)
+{
+    float d;
+    asm("max.NaN.abs.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
+}
+__device__ __forceinline__ float min3abs(float a, float b, float c)
+{
+    float d;
+    asm("min.abs.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
+}
+
+// a packed FP64 spinor's words, and the biased exponents of its largest and
+// smallest component
+struct FixRaw {
+    uint4 w[12];
+    int emax, emin;
+    __device__ __forceinline__ void load(const Spinor64 &in, int i)
+    {
+        const uint4 *q = reinterpret_cast<const uint4 *>(in.at(i));
+#pragma unroll
+        for (int k = 0; k < 12; ++k) w[k] = __ldg(q + ((size_t)k << in.lvb));
+    }
+    // from the thread's staging slots
+    __device__ __forceinline__ void load_staged(const int4 *slot)
+    {
+#pragma unroll
+        for (int k = 0; k < 12; ++k) {
+            const int4 v = slot[k * FIX_THREADS];
+            w[k] = make_uint4(v.x, v.y, v.z, v.w);
+        }
+    }
+    __device__ __forceinline__ void range()
+    {
+        float mx = fabsf(__uint_as_float(w[0].y)), mn = mx;
+#pragma unroll
+        for (int k = 0; k < 12; ++k) {
+            mx = max3abs(mx, __uint_as_float(w[k].y), __uint_as_float(w[k].w));
+            mn = min3abs(mn, __uint_as_float(w[k].y), __uint_as_float(w[k].w));
+        }
+        emax = __float_as_int(mx) >> 20;
+        emin = __float_as_int(mn) >> 20;
+    }
+};
+
+// Q = x 2^(60 - E) for a double x with |x| < 2^E, K = E's biased exponent + 4,
+// valid while K - (x's biased exponent) < 32.
+// Negative values come out one unit (2^-60) low: the sign is applied as a
+// one's complement.  neg = ~0 negates x.
+__device__ __forceinline__ fix_t fix_from(uint32_t lo, uint32_t hi, int K, uint32_t neg)
+{
+    const uint32_t u = __funnelshift_l(lo, hi, 11) | 0x80000000u, v = lo << 11;
+    const int s = K - (int)(hi >> 20);  // the sign bit adds a multiple of 32
+    const uint32_t sm = (uint32_t)((int)hi >> 31);
+    const uint32_t ql = __funnelshift_r(v, u, s) ^ sm ^ neg;
+    const uint32_t qh = __funnelshift_r(u, 0u, s) ^ sm ^ neg;
+    return (fix_t)(((unsigned long long)qh << 32) | ql);
+}
+
+// component k of the site in units of 2^(E - 60), K = E + 4
+__device__ __forceinline__ Cx<fix_t> fix_component(const FixRaw &r, int k, int K, uint32_t neg = 0)
+{
+    return {fix_from(r.w[k].x, r.w[k].y, K, neg), fix_from(r.w[k].z, r.w[k].w, K, neg)};
+}
+
+// every component of the site is zero (emax == 0 leaves zeros and denormals)
+__device__ __forceinline__ bool fix_all_zero(const FixRaw &r)
+{
+    if (r.emax != 0) return false;
+    uint32_t any = 0;
+#pragma unroll
+    for (int k = 0; k < 12; ++k) any |= r.w[k].x | r.w[k].z | ((r.w[k].y | r.w[k].w) & 0x7fffffffu);
+    return any == 0;
+}
+
+// the site's components can be converted to units of 2^(E - 60): all of them
+// nonzero, in range and above 2^-27 of 2^E
+__device__ __forceinline__ bool fix_in_range(const FixRaw &r, int E)
+{
+    return r.emax < FIX_EMAX && r.emax >= FIX_EMIN && E + 4 - r.emin < 32;
+}
+
+// limbs with a balanced low part
+__device__ __forceinline__ void fix_limbs(fix_t q, int &hi, int &lo)
+{
+    lo = (int)q;
+    hi = (int)((uint32_t)((unsigned long long)q >> 32) + ((uint32_t)lo >> 31));
+    asm("" : "+r"(lo), "+r"(hi));  // 32-bit numbers of unknown origin (above)
+}
+
+// hh + mid 2^-32 in units of hh, rounded down
+__device__ __forceinline__ fix_t fix_join(fix_t hh, fix_t mid) { return mac64((int)(mid >> 32), 1, hh); }
+
+// (a, b) + sgn P (l0, l1) with P the spin map of direction MU: the projected
+// half spinor of one colour
+template <int MU, int SGN>
+__device__ __forceinline__ void fix_project(Cx<fix_t> &a, Cx<fix_t> &b, Cx<fix_t> l0, Cx<fix_t> l1)
+{
+    Cx<fix_t> o0, o1;
+    isigma<MU>(l0, l1, o0, o1);
+    a = SGN > 0 ? a - o0 : a + o0;
+    b = SGN > 0 ? b - o1 : b + o1;
+}
+
+// the lower spins of one colour reconstructed from (w0, w1), as reconstruct_add
+template <int MU, int SGN>
+__device__ __forceinline__ void fix_reconstruct(Cx<fix_t> &a, Cx<fix_t> &b, Cx<fix_t> w0, Cx<fix_t> w1)
+{
+    Cx<fix_t> o0, o1;
+    isigma<MU>(w0, w1, o0, o1);
+    if ((MU == 3) == (SGN > 0)) {
+        a = a - o0;
+        b = b - o1;
+    } else {
+        a = a + o0;
+        b = b + o1;
+    }
+}
+
+// a direction known at run time (the same for every thread), as a switch over
+// its spin maps: m = 2 mu + (projector 1 + gamma)
+#define MGC_FIX_SWITCH(m, CALL)        \
+    switch (m) {                       \
+    case 0: CALL(0, -1); break;        \
+    case 1: CALL(0, +1); break;        \
+    case 2: CALL(1, -1); break;        \
+    case 3: CALL(1, +1); break;        \
+    case 4: CALL(2, -1); break;        \
+    case 5: CALL(2, +1); break;        \
+    case 6: CALL(3, -1); break;        \
+    default: CALL(3, +1); break;       \
+    }
+
+// The projected half spinor of direction m (above) from the spinor in the
+// staging slots (negated where `flip`, conjugated where `back`), as limbs; raises E (and shifts acc down) where the neighbour
+// exceeds it; FIX_LEAVE when the site needs FP64.
+enum { FIX_LEAVE, FIX_ZERO, FIX_HOP };
+__device__ __forceinline__ int fix_half_spinor(const int4 *slot, int m, bool back, bool flip, Cx<fix_t> acc[12],
+                                                int &E, int h1[12], int h0[12])
+{
+    FixRaw r;
+    r.load_staged(slot);
+    r.range();
+    if (r.emax > E) {
+        const int d = min(r.emax - E, 63);
+        E = r.emax;
+#pragma unroll
+        for (int k = 0; k < 12; ++k) acc[k] = Cx<fix_t>{acc[k].r >> d, acc[k].i >> d};
+    }
+    if (!fix_in_range(r, E)) return fix_all_zero(r) ? FIX_ZERO : FIX_LEAVE;
+    const int K = E + 4;
+    const uint32_t fm = flip ? ~0u : 0u;
+    const fix_t bm = back ? -1 : 0;
+    // colour by colour, so that few 64-bit intermediates live at a time
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        Cx<fix_t> a = fix_component(r, k, K, fm), b = fix_component(r, 3 + k, K, fm);
+        const Cx<fix_t> l0 = fix_component(r, 6 + k, K, fm), l1 = fix_component(r, 9 + k, K, fm);
+#define MGC_FIX_CALL(MU, SGN) fix_project<MU, SGN>(a, b, l0, l1)
+        MGC_FIX_SWITCH(m, MGC_FIX_CALL)
+#undef MGC_FIX_CALL
+        a.i ^= bm;
+        b.i ^= bm;
+        fix_limbs(a.r, h1[2 * k], h0[2 * k]);
+        fix_limbs(a.i, h1[2 * k + 1], h0[2 * k + 1]);
+        fix_limbs(b.r, h1[2 * k + 6], h0[2 * k + 6]);
+        fix_limbs(b.i, h1[2 * k + 7], h0[2 * k + 7]);
+    }
+    return FIX_HOP;
+}
+
+// acc += the hop of direction m from its projected half spinor h (conjugated for
+// a backward hop) and the link in the staging slots.  U^dagger h is the conjugate
+// of U^T conj(h): the backward hop reads the transposed entries and negates the
+// imaginary parts on the way in and out, as one's complements.
+__device__ __forceinline__ void fix_hop(const int4 *slot, int m, bool back, const int h1[12], const int h0[12],
+                                        Cx<fix_t> acc[12])
+{
+    const int sa = (back ? 1 : 3) * FIX_THREADS, sb = (back ? 3 : 1) * FIX_THREADS;
+    const fix_t bm = back ? -1 : 0;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        fix_t hr[2], hi[2], mr[2], mi[2];
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            const int4 u = slot[a * sa + b * sb];
+            const int n1 = fix_neg(u.z), n0 = fix_neg(u.w);
+#pragma unroll
+            for (int s = 0; s < 2; ++s) {
+                const int k = 2 * (3 * s + b);
+                const int x1 = h1[k], x0 = h0[k], y1 = h1[k + 1], y0 = h0[k + 1];
+                hr[s] = mac64(n1, y1, b ? mac64(u.x, x1, hr[s]) : mul64(u.x, x1));
+                mr[s] = mac64(u.y, x1, b ? mac64(u.x, x0, mr[s]) : mul64(u.x, x0));
+                mr[s] = mac64(n0, y1, mac64(n1, y0, mr[s]));
+                hi[s] = mac64(u.z, x1, b ? mac64(u.x, y1, hi[s]) : mul64(u.x, y1));
+                mi[s] = mac64(u.y, y1, b ? mac64(u.x, y0, mi[s]) : mul64(u.x, y0));
+                mi[s] = mac64(u.w, x1, mac64(u.z, x0, mi[s]));
+            }
+        }
+        const Cx<fix_t> w0 = {fix_join(hr[0], mr[0]), fix_join(hi[0], mi[0]) ^ bm};
+        const Cx<fix_t> w1 = {fix_join(hr[1], mr[1]), fix_join(hi[1], mi[1]) ^ bm};
+        acc[a] = acc[a] + w0;
+        acc[3 + a] = acc[3 + a] + w1;
+#define MGC_FIX_CALL(MU, SGN) fix_reconstruct<MU, SGN>(acc[6 + a], acc[9 + a], w0, w1)
+        MGC_FIX_SWITCH(m, MGC_FIX_CALL)
+#undef MGC_FIX_CALL
+    }
+}
+
+// the neighbour of hop d (mu = d / 2, backward when odd), and whether the hop
+// carries the boundary sign
+__device__ __forceinline__ int fix_neighbour(const Geom &g, const int c[4], int d, bool &flip)
+{
+    const int step = d & 1 ? -1 : 1;
+    int n[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        int v = c[k] + (k == (d >> 1) ? step : 0);
+        const bool lo = v < 0, hi = v >= g.L[k];
+        v = lo ? v + g.L[k] : (hi ? 0 : v);
+        if (k == 3) flip = (lo || hi) && g.tbc < 0;
+        n[k] = v;
+    }
+    return site_index(g, n);
+}
+
+// acc = C/kappa psi in the sum's unit: the products' unit times 2^L, L <= 4
+__device__ __forceinline__ void fix_clover(const FixClover &C, int i, const FixRaw &r, int K, int L,
+                                           Cx<fix_t> acc[12])
+{
+    const int4 *cp = C.at(i);
+#pragma unroll
+    for (int chi = 0; chi < 2; ++chi) {
+        int v1[12], v0[12];
+        fix_t hh[12], mid[12];
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            const Cx<fix_t> q = fix_component(r, 6 * chi + k, K);
+            fix_limbs(q.r, v1[2 * k], v0[2 * k]);
+            fix_limbs(q.i, v1[2 * k + 1], v0[2 * k + 1]);
+        }
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const int4 d = __ldg(cp + ((size_t)(18 * chi + k) << C.lvb));
+#pragma unroll
+            for (int z = 0; z < 2; ++z) {
+                hh[4 * k + z] = mul64(d.x, v1[4 * k + z]);
+                mid[4 * k + z] = mac64(d.x, v0[4 * k + z], mul64(d.y, v1[4 * k + z]));
+                hh[4 * k + 2 + z] = mul64(d.z, v1[4 * k + 2 + z]);
+                mid[4 * k + 2 + z] = mac64(d.z, v0[4 * k + 2 + z], mul64(d.w, v1[4 * k + 2 + z]));
+            }
+        }
+        int k = 3;
+#pragma unroll
+        for (int a = 1; a < 6; ++a)
+#pragma unroll
+            for (int b = 0; b < a; ++b) {
+                const int4 l = __ldg(cp + ((size_t)(18 * chi + k++) << C.lvb));
+                const int n1 = fix_neg(l.z), n0 = fix_neg(l.w);
+                // o[a] += L v[b], o[b] += conj(L) v[a]
+#pragma unroll
+                for (int t = 0; t < 2; ++t) {
+                    const int o = 2 * (t ? b : a), x = 2 * (t ? a : b);
+                    const int s1 = t ? l.z : n1, s0 = t ? l.w : n0;  // sign of the (im, im) product
+                    const int c1 = t ? n1 : l.z, c0 = t ? n0 : l.w;
+                    hh[o] = mac64(l.x, v1[x], hh[o]);
+                    mid[o] = mac64(l.x, v0[x], mid[o]);
+                    mid[o] = mac64(l.y, v1[x], mid[o]);
+                    hh[o] = mac64(s1, v1[x + 1], hh[o]);
+                    mid[o] = mac64(s1, v0[x + 1], mid[o]);
+                    mid[o] = mac64(s0, v1[x + 1], mid[o]);
+                    hh[o + 1] = mac64(l.x, v1[x + 1], hh[o + 1]);
+                    mid[o + 1] = mac64(l.x, v0[x + 1], mid[o + 1]);
+                    mid[o + 1] = mac64(l.y, v1[x + 1], mid[o + 1]);
+                    hh[o + 1] = mac64(c1, v1[x], hh[o + 1]);
+                    mid[o + 1] = mac64(c1, v0[x], mid[o + 1]);
+                    mid[o + 1] = mac64(c0, v1[x], mid[o + 1]);
+                }
+            }
+#pragma unroll
+        for (int m = 0; m < 12; ++m) {
+            const fix_t y = fix_join(hh[m], mid[m]);
+            fix_t r;
+            if (L >= 0) {  // up to four bits of the middle sum below hh's unit
+                const uint32_t lo = __funnelshift_l((uint32_t)mid[m], (uint32_t)y, L);
+                const uint32_t hi = __funnelshift_l((uint32_t)y, (uint32_t)(y >> 32), L);
+                r = (fix_t)(((unsigned long long)hi << 32) | lo);
+            } else {
+                r = y >> min(-L, 63);
+            }
+            (m & 1 ? acc[6 * chi + (m >> 1)].i : acc[6 * chi + (m >> 1)].r) = r;
+        }
+    }
+}
+
+// (D psi)(x) with FP64 instructions, for the sites the fixed-point path leaves
+template <bool DAG>
+__device__ __noinline__ void fix_fallback(const Geom &g, int i, const Spinor64 &in, const Spinor64 &out,
+                                          const Gauge64 &U, const Clover64 &C, double kappa)
+{
+    int c[4];
+    site_coords(g, i, c);
+    const Spinor64 one[1] = {in};
+    Cx<double> o[1][12];
+    dirac_site_pair<DAG, 1>(g, c, i, one, 1, U, C, kappa, o);
+    out.store(i, o[0]);
+}
+
+// out(i) = (D psi)(i) in fixed point; false (nothing stored) when the site needs
+// FP64.  `slots` is the thread's column of the block's staging slots.  One copy
+// of the hop's code serves all eight: unrolled per direction the kernel is 12,600
+// instructions long and waits on instruction fetch for half its time (1060 us on
+// 24^3 x 48).  The next hop's spinor and link are copied to shared memory while
+// this hop's products run; without that, loads were the first stall (433 us).
+template <bool DAG>
+__device__ __forceinline__ bool fix_dirac_site(const Geom &g, int i, const Spinor64 &in, const Spinor64 &out,
+                                               const FixLinks &U, const FixClover &C, double kappa, int4 *slots)
+{
+    int4 *const ls = slots + FIX_SPINOR_SLOTS * FIX_THREADS;
+    auto copy_spinor = [&](int j) {
+        const double2 *q = in.at(j);
+#pragma unroll
+        for (int k = 0; k < FIX_SPINOR_SLOTS; ++k) fix_copy16(slots + k * FIX_THREADS, q + ((size_t)k << in.lvb));
+    };
+    auto copy_link = [&](int d, int j) {
+        const int4 *q = U.at(d & 1 ? j : i, d >> 1);
+#pragma unroll
+        for (int k = 0; k < FIX_LINK_SLOTS; ++k) fix_copy16(ls + k * FIX_THREADS, q + ((size_t)k << U.lvb));
+    };
+    int c[4];
+    site_coords(g, i, c);
+    bool flip;
+    int j = fix_neighbour(g, c, 0, flip);
+    copy_spinor(j);
+    fix_commit();
+    copy_link(0, j);
+    fix_commit();
+
+    Cx<fix_t> acc[12];
+    int E;
+    int state = FIX_HOP, zeros = 0;
+    {
+        FixRaw r;
+        r.load(in, i);
+        r.range();
+        const int eC = __ldg(C.e + i);
+        const int ep = max(r.emax, FIX_EMIN);
+        E = ep + max(0, eC - 2);
+        if (fix_in_range(r, ep)) {
+            fix_clover(C, i, r, ep + 4, eC + 2 + ep - E, acc);
+        } else {
+            state = fix_all_zero(r) ? FIX_ZERO : FIX_LEAVE;
+#pragma unroll
+            for (int k = 0; k < 12; ++k) acc[k] = Cx<fix_t>{0, 0};
+        }
+    }
+    // H enters with a minus sign: sum H - C/kappa, and -kappa at the end.  The
+    // eight hops' truncation is half a unit each on average.
+#pragma unroll
+    for (int k = 0; k < 12; ++k) acc[k] = Cx<fix_t>{4 - acc[k].r, 4 - acc[k].i};
+#pragma unroll 1
+    for (int d = 0; d < 8 && state != FIX_LEAVE; ++d) {
+        const int m = (d & ~1) + (int)((bool)(d & 1) != DAG);
+        int h1[12], h0[12];
+        fix_wait<1>();  // this hop's spinor (its link may be in flight)
+        state = fix_half_spinor(slots, m, d & 1, flip, acc, E, h1, h0);
+        if (d < 7) {
+            // every slot has been read: the test above depends on all of them
+            j = fix_neighbour(g, c, d + 1, flip);
+            copy_spinor(j);
+        }
+        fix_commit();
+        fix_wait<1>();  // this hop's link
+        if (state == FIX_HOP) fix_hop(ls, m, d & 1, h1, h0, acc);
+        else ++zeros;
+        if (d < 7) copy_link(d + 1, j);
+        fix_commit();
+    }
+    fix_wait<0>();
+    if (state == FIX_LEAVE) return false;
+    if (zeros) {  // their half units; nine zero sites give an exact zero
+#pragma unroll
+        for (int k = 0; k < 12; ++k) acc[k] = Cx<fix_t>{acc[k].r - (zeros >> 1), acc[k].i - (zeros >> 1)};
+    }
+    const double sc = -kappa * __hiloint2double((E - 55) << 20, 0);
+    Cx<double> o[12];
+#pragma unroll
+    for (int k = 0; k < 12; ++k)
+        o[k] = Cx<double>{sc * __ll2double_rn(acc[k].r), sc * __ll2double_rn(acc[k].i)};
+    out.store(i, o);
+    return true;
+}
+
+}  // namespace mgc

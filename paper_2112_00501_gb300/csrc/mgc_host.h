@@ -21,6 +21,7 @@ struct mgc_lattice_s {
 struct mgc_gauge_s {
     mgc_lattice_s *lat;
     double2 *U64;  // packed FP64, 18 reals per link
+    int4 *UQ;      // the links in fixed point for the FP64 operator (NULL unless near unitary)
     void *U32;     // packed FP32 at compress (NULL when prec == 64)
     void *U16;     // packed FP16 at compress (NULL unless prec == 16)
     int prec;      // storage precision: 64, 32 or 16
@@ -36,6 +37,8 @@ struct mgc_clover_s {
     double kappa, csw;
     double2 *C64;   // packed FP64 clover C
     double2 *Ci64;  // packed FP64 C^-1
+    int4 *CQ;       // C/kappa in fixed point and its site exponents (NULL: D runs on FP64 units)
+    int *CE;
     void *C32;      // packed FP32 C (NULL when prec == 64)
     void *C16;      // packed FP16 C followed by its per-site scales (prec == 16)
     float *C16_sc;
@@ -97,6 +100,9 @@ int launch_pack(const Geom &g, int prec, int nrhs, const double *canon, void *pa
 int launch_unpack(const Geom &g, int prec, int nrhs, const void *packed, double *canon, cudaStream_t s);
 int launch_convert(const Geom &g, int nrhs, int pin, const void *in, int pout, void *out, cudaStream_t s);
 int launch_gauge_pack(const Geom &g, const double *canon_dev, int prec, int compress, void *out, cudaStream_t s);
+// fixed-point copies of the links and of C/kappa; *d_bad is set when a field is out of their range
+int launch_fix_links(const Geom &g, const double2 *U64, int4 *out, int *d_bad, cudaStream_t s);
+int launch_fix_clover(const Geom &g, const double2 *C64, double kappa, int4 *out, int *ex, int *d_bad, cudaStream_t s);
 int launch_dirac(const mgc_clover_s *op, int prec, bool dag, const void *in, void *out, int nrhs,
                  cudaStream_t s);
 // w = D z with the FP32 operator for an FP16 z (FP32 result)

@@ -1,0 +1,121 @@
+"""The FP64 operator's block fixed-point path: its error, the fields it leaves
+to FP64 instructions, and the batched operator's agreement with it.
+
+Bound: a component is off by at most the fixed-point truncation, a few units of
+2^-54 of the largest |psi| near the site against |D psi| of the same order, and
+the result's own rounding 2^-53; 6e-16 in the 2-norm leaves a factor two over
+both and the reference's own error, the oracle's FP64 sum, good to 2e-16.
+"""
+import numpy as np
+import pytest
+
+from helpers import fields, rel
+from oracle import oracle as O
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+def _op(name, U=None, kappa=None, tbc=-1):
+    from paper_2112_00501_gb300 import api
+
+    dims, block, eps, kap, csw, U0, psi = fields(name)
+    lat = api.Lattice(dims, block, tbc)
+    g = api.Gauge(lat, torch.from_numpy(U0 if U is None else U).cuda(), storage_prec=64)
+    return api.CloverOperator(g, kap if kappa is None else kappa, csw)
+
+
+def _scaled(psi, p):
+    return np.ldexp(np.ascontiguousarray(psi).view(np.float64), p).view(np.complex128)
+
+
+def _check(name, psi, tol=6e-16, U=None, kappa=None, dagger=False, p=0):
+    dims, block, eps, kap, csw, U0, _ = fields(name)
+    U, kappa = U0 if U is None else U, kap if kappa is None else kappa
+    got = _op(name, U, kappa).D(torch.from_numpy(_scaled(psi, p)).cuda(), prec=64, dagger=dagger).cpu().numpy()
+    got = _scaled(got, -p)
+    ref = O.dirac(dims, -1, kappa, U, O.clover(dims, kappa, csw, U), psi, dagger=dagger)
+    assert rel(got, ref) < tol
+    return got, ref
+
+
+@pytest.mark.parametrize("name", ["c0_4^4", "ragged_8x4x12x8", "mid_8^4"])
+@pytest.mark.parametrize("dagger", [False, True])
+@pytest.mark.parametrize("kappa", [0.01, 0.13, -0.13, 0.8, 70.0])  # 0.01 and 70 run on FP64 instructions
+def test_error(name, dagger, kappa):
+    _check(name, fields(name)[6], kappa=kappa, dagger=dagger)
+
+
+@pytest.mark.parametrize("p", [-1000, -900, -890, -400, 400, 955, 964])
+def test_scales_of_the_whole_field(p):
+    _check("ragged_8x4x12x8", fields("ragged_8x4x12x8")[6], p=p)
+
+
+@pytest.mark.parametrize("kind", ["sites", "neighbours", "components", "zeros", "point", "one_spin"])
+def test_wide_and_sparse_fields(kind):
+    """Component-wise at sites that see only one scale, 2-norm elsewhere."""
+    name = "mid_8^4"
+    psi = fields(name)[6].copy()
+    r = np.random.default_rng(3)
+    V = psi.shape[0]
+    if kind == "sites":  # neighbours up to 2^24 apart: inside the fixed-point range
+        psi *= np.exp2(r.integers(-12, 13, V))[:, None, None]
+    if kind == "neighbours":  # beyond it
+        psi *= np.exp2(r.integers(-60, 61, V))[:, None, None]
+    if kind == "components":
+        psi *= np.exp2(r.integers(-40, 41, psi.shape))
+    if kind == "zeros":
+        psi[r.random(V) < 0.5] = 0
+    if kind == "point":
+        psi[:] = 0
+        psi[77, 2, 1] = 1.5 - 0.25j
+    if kind == "one_spin":
+        psi[:, 1:] = 0
+    got, ref = _check(name, psi)
+    assert np.array_equal(got == 0, ref == 0) or kind in ("sites", "neighbours", "components")
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf])
+def test_non_finite_propagates(bad):
+    name = "mid_8^4"
+    dims, block, eps, kappa, csw, U, psi = fields(name)
+    psi = psi.copy()
+    psi[100, 1, 2] = bad
+    got = _op(name).D(torch.from_numpy(psi).cuda(), prec=64).cpu().numpy()
+    clean = O.dirac(dims, -1, kappa, U, O.clover(dims, kappa, csw, U), fields(name)[6])
+    hit = ~np.isfinite(got).all(axis=(1, 2))
+    assert hit.sum() == 9 and hit[100]  # the site and its eight neighbours
+    assert rel(got[~hit], clean[~hit]) < 6e-16
+
+
+def test_links_that_are_not_unitary():
+    name = "mid_8^4"
+    U = fields(name)[5].copy()
+    U[5, 2] *= 1.01  # no fixed-point copy: FP64 instructions
+    _check(name, fields(name)[6], U=U)
+    U = fields(name)[5].copy()
+    U[5, 2] *= 1 + 1e-5  # within the copy's bound
+    _check(name, fields(name)[6], U=U)
+
+
+def test_batch_is_bit_identical():
+    """A batch of one lattice with a fixed-point copy and one without."""
+    from paper_2112_00501_gb300 import api
+
+    name = "mid_8^4"
+    V = fields(name)[6].shape[0]
+    bent = fields(name)[5].copy()
+    bent[5, 2] *= 1.01
+    ops = [_op(name), _op(name, bent)]
+    g = torch.Generator(device="cuda").manual_seed(5)
+    xs = [torch.view_as_complex(torch.randn((n, V, 4, 3, 2), dtype=torch.float64, device="cuda", generator=g))
+          for n in (3, 1)]
+    ps = [op.lattice.pack(x, 64) for op, x in zip(ops, xs)]
+    batch = api.Batch(ops, [3, 1])
+    for dagger in (False, True):
+        for fast in (0, 1):
+            batch.set_shape(64, 1, 128, fast, 0)
+            out = batch.apply_D(ps, 64, dagger=dagger)
+            for op, p, n, o in zip(ops, ps, (3, 1), out):
+                assert torch.equal(o, (op.apply_Ddag if dagger else op.apply_D)(p, 64, n))

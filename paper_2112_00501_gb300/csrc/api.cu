@@ -192,14 +192,11 @@ int mgc_gauge_create(mgc_lattice_t lat, const double *U, int on_device, int stor
     G->compress = (storage_prec == 64) ? 18 : compress;
     int st = MGC_OK;
     double *d_err = nullptr;
-    int *d_bad = nullptr;
     auto bail = [&](int code) {
         cudaFree(canon);
         cudaFree(d_err);
-        cudaFree(d_bad);
         if (code != MGC_OK) {
             cudaFree(G->U64);
-            cudaFree(G->UQ);
             cudaFree(G->U32);
             cudaFree(G->U16);
             delete G;
@@ -230,14 +227,6 @@ int mgc_gauge_create(mgc_lattice_t lat, const double *U, int on_device, int stor
     GCUDA(cudaMalloc(&G->U64, gauge_bytes(g, 64, 18)));
     st = launch_gauge_pack(g, src, 64, 18, G->U64, s);
     if (st) return bail(st);
-    // the fixed-point copy of the FP64 operator; kept where every link is near unitary
-    GCUDA(cudaMalloc(&d_bad, sizeof(int)));
-    GCUDA(cudaMemsetAsync(d_bad, 0, sizeof(int), s));
-    GCUDA(cudaMalloc(&G->UQ, gauge_bytes(g, 64, 18)));
-    st = launch_fix_links(g, G->U64, G->UQ, d_bad, s);
-    if (st) return bail(st);
-    int bad = 0;
-    GCUDA(cudaMemcpyAsync(&bad, d_bad, sizeof(int), cudaMemcpyDeviceToHost, s));
     if (storage_prec <= 32) {
         GCUDA(cudaMalloc(&G->U32, gauge_bytes(g, 32, G->compress)));
         st = launch_gauge_pack(g, src, 32, G->compress, G->U32, s);
@@ -250,10 +239,6 @@ int mgc_gauge_create(mgc_lattice_t lat, const double *U, int on_device, int stor
     }
     GCUDA(cudaStreamSynchronize(s));
 #undef GCUDA
-    if (bad) {
-        cudaFree(G->UQ);
-        G->UQ = nullptr;
-    }
     *out = G;
     return bail(MGC_OK);
 }
@@ -262,11 +247,19 @@ int mgc_gauge_destroy(mgc_gauge_t g)
 {
     if (!g) return MGC_OK;
     cudaFree(g->U64);
-    cudaFree(g->UQ);
     cudaFree(g->U32);
     cudaFree(g->U16);
     delete g;
     return MGC_OK;
+}
+
+static void free_fix(mgc_clover_s *op)
+{
+    cudaFree(op->UQ);
+    cudaFree(op->CQ);
+    cudaFree(op->CE);
+    op->UQ = op->CQ = nullptr;
+    op->CE = nullptr;
 }
 
 int mgc_clover_create(mgc_gauge_t g, double kappa, double csw, void *stream, mgc_clover_t *out)
@@ -284,8 +277,7 @@ int mgc_clover_create(mgc_gauge_t g, double kappa, double csw, void *stream, mgc
         if (code != MGC_OK) {
             cudaFree(op->C64);
             cudaFree(op->Ci64);
-            cudaFree(op->CQ);
-            cudaFree(op->CE);
+            free_fix(op);
             cudaFree(op->C32);
             cudaFree(op->C16);
             cudaFree(op->Ci32);
@@ -304,17 +296,25 @@ int mgc_clover_create(mgc_gauge_t g, double kappa, double csw, void *stream, mgc
     CCUDA(cudaMemsetAsync(op->d_status, 0, sizeof(int), s));
     CCUDA(cudaMalloc(&op->C64, clover_bytes(geo, 64)));
     CCUDA(cudaMalloc(&op->Ci64, clover_bytes(geo, 64)));
-    CCUDA(cudaMalloc(&d_bad, 2 * sizeof(int)));
-    CCUDA(cudaMemsetAsync(d_bad, 0, 2 * sizeof(int), s));
+    CCUDA(cudaMalloc(&d_bad, 3 * sizeof(int)));
+    CCUDA(cudaMemsetAsync(d_bad, 0, 3 * sizeof(int), s));
     int st = launch_clover_build(geo, g->U64, kappa, csw, op->C64, op->Ci64, d_bad, s);
     if (st) return bail(st);
-    // C/kappa in fixed point for the FP64 operator, for hopping parameters and
-    // clover terms of ordinary size
-    const bool fix = g->UQ && fabs(kappa) >= 0x1p-6 && fabs(kappa) <= 0x1p6;
-    if (fix) {
-        CCUDA(cudaMalloc(&op->CQ, clover_bytes(geo, 64)));
-        CCUDA(cudaMalloc(&op->CE, (size_t)geo.V * sizeof(int)));
-        st = launch_fix_clover(geo, op->C64, kappa, op->CQ, op->CE, d_bad + 1, s);
+    // fixed-point copies for the FP64 operator, for hopping parameters of ordinary
+    // size and where there is room for them (it runs without)
+    const double ks = std::frexp(kappa, &op->fix_ek);
+    if (fabs(kappa) >= 0x1p-16 && fabs(kappa) <= 0x1p16) {
+        if (cudaMalloc(&op->UQ, gauge_bytes(geo, 64, 18)) != cudaSuccess ||
+            cudaMalloc(&op->CQ, clover_bytes(geo, 64)) != cudaSuccess ||
+            cudaMalloc(&op->CE, (size_t)geo.V * sizeof(int2)) != cudaSuccess) {
+            (void)cudaGetLastError();
+            free_fix(op);
+        }
+    }
+    if (op->CQ) {
+        st = launch_fix_links(geo, g->U64, ks, op->UQ, d_bad + 1, s);
+        if (st) return bail(st);
+        st = launch_fix_clover(geo, op->C64, op->fix_ek, op->CQ, op->CE, d_bad + 1, s);
         if (st) return bail(st);
     }
     // C and C^-1 (the latter for the clover-preconditioned operator A = C^-1 D)
@@ -337,17 +337,13 @@ int mgc_clover_create(mgc_gauge_t g, double kappa, double csw, void *stream, mgc
         st = launch_clover_lowprec(geo, op->Ci64, 16, op->Ci16, s);
         if (st) return bail(st);
     }
-    int bad[2] = {0, 0};
-    CCUDA(cudaMemcpyAsync(bad, d_bad, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
+    int bad[3] = {0, 0, 0};
+    CCUDA(cudaMemcpyAsync(bad, d_bad, 3 * sizeof(int), cudaMemcpyDeviceToHost, s));
     CCUDA(cudaStreamSynchronize(s));
 #undef CCUDA
     if (bad[0]) return bail(fail(MGC_ERR_BREAKDOWN, "singular clover block"));
-    if (bad[1]) {
-        cudaFree(op->CQ);
-        cudaFree(op->CE);
-        op->CQ = nullptr;
-        op->CE = nullptr;
-    }
+    if (bad[1]) free_fix(op);
+    op->fix_room = bad[2];
     *out = op;
     return bail(MGC_OK);
 }
@@ -358,8 +354,7 @@ int mgc_clover_destroy(mgc_clover_t op)
     free_work(op);
     cudaFree(op->C64);
     cudaFree(op->Ci64);
-    cudaFree(op->CQ);
-    cudaFree(op->CE);
+    free_fix(op);
     cudaFree(op->C32);
     cudaFree(op->C16);
     cudaFree(op->Ci32);

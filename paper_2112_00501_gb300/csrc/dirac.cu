@@ -195,9 +195,18 @@ __device__ __forceinline__ int2 fix_store(fix_t q)
     return make_int2(hi, max(lo, -0x7fffffff));
 }
 
-// The links in units of 2^-60; *bad is set unless the rows and columns of every
-// link have norm 1 to 1e-3, which bounds the operator's sums.
-__global__ void k_fix_links(Geom g, Gauge64 U, int4 *__restrict__ out, int *bad)
+// a b 2^60
+__device__ __forceinline__ int2 fix_product(double a, double b)
+{
+    const double hi = a * b, lo = fma(a, b, -hi);
+    const fix_t t = __double2ll_rn(hi * 0x1p60);
+    return fix_store(t + __double2ll_rn((hi * 0x1p60 - (double)t) + lo * 0x1p60));
+}
+
+// The links times ks (|ks| <= 1) in units of 2^-60, the product formed with its
+// remainder; *bad is set unless the rows and columns of every link have norm 1 to
+// 1e-3, which bounds the operator's sums.
+__global__ void k_fix_links(Geom g, Gauge64 U, double ks, int4 *__restrict__ out, int *bad)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= g.V) return;
@@ -214,64 +223,84 @@ __global__ void k_fix_links(Geom g, Gauge64 U, int4 *__restrict__ out, int *bad)
     }
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
-        const int2 r = fix_store(__double2ll_rn(u[k].r * 0x1p60)), m = fix_store(__double2ll_rn(u[k].i * 0x1p60));
+        const int2 r = fix_product(u[k].r, ks), m = fix_product(u[k].i, ks);
         o[(size_t)k << g.lvb] = make_int4(r.x, r.y, m.x, m.y);
     }
     if (!fine) atomicOr(bad, 1);
 }
 
-// C/kappa in units of 2^(e - 58) with the site's exponent e, |C/kappa| < 2^e.
-// The quotient is formed with its remainder, so the 58 bits are C's own.
-__global__ void k_fix_clover(Geom g, Clover64 C, double kappa, int4 *__restrict__ out, int *__restrict__ ex, int *bad)
+// C in units of 2^(e + ek - 60) with the site's exponent e, |C| < 2^(e + ek) and a
+// row's absolute sum below four times that, and the bits room that the sum's unit leaves for it: a row's absolute sum is below
+// 2^(5 + room + ek).
+__global__ void k_fix_clover(Geom g, Clover64 C, int ek, int4 *__restrict__ out, int2 *__restrict__ ex, int *bad)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= g.V) return;
     const double2 *q = C.p + ((size_t)(i >> g.lvb) * 36 << g.lvb) + (i & ((1 << g.lvb) - 1));
-    double m = 0;
+    double m = 0, row = 0;
     bool fine = true;
-    for (int k = 0; k < 36; ++k) {
-        const double2 v = q[(size_t)k << g.lvb];
-        m = fmax(m, fmax(fabs(v.x), fabs(v.y)));
-        fine = fine && isfinite(v.x) && isfinite(v.y);
+#pragma unroll
+    for (int chi = 0; chi < 2; ++chi) {
+        double sum[6];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const double2 v = q[(size_t)(18 * chi + k) << g.lvb];
+            sum[2 * k] = fabs(v.x);
+            sum[2 * k + 1] = fabs(v.y);
+            m = fmax(m, fmax(fabs(v.x), fabs(v.y)));
+        }
+        int k = 3;
+#pragma unroll
+        for (int a = 1; a < 6; ++a)
+#pragma unroll
+            for (int b = 0; b < a; ++b) {
+                const double2 v = q[(size_t)(18 * chi + k++) << g.lvb];
+                const double t = fabs(v.x) + fabs(v.y);
+                sum[a] += t;
+                sum[b] += t;
+                m = fmax(m, fmax(fabs(v.x), fabs(v.y)));
+            }
+#pragma unroll
+        for (int a = 0; a < 6; ++a) {
+            fine = fine && isfinite(sum[a]);  // NaN entries too, which fmax drops
+            row = fmax(row, sum[a]);
+        }
     }
-    const int e = ilogb(m / kappa) + 2;  // one to spare for the quotient's rounding
-    if (!fine || m == 0 || e < -16 || e > 16) {
+    if (!fine || m < 0x1p-16 || row > 0x1p16) {
         atomicOr(bad, 1);
         return;
     }
-    ex[i] = e;
-    const double s = ldexp(1.0, 58 - e);
+    const int lrow = ilogb(row * (1.0 + 0x1p-40)) + 1;
+    const int e = max(ilogb(m) + 1, lrow - 2) - ek, room = max(0, lrow - ek - 5);
+    ex[i] = make_int2(e, room);
+    atomicMax(bad + 1, room);
+    const double s = ldexp(1.0, 60 - e - ek);
     int4 *o = out + ((size_t)(i >> g.lvb) * 36 << g.lvb) + (i & ((1 << g.lvb) - 1));
-    auto one = [&](double c) {
-        const double hi = c / kappa, lo = fma(-hi, kappa, c) / kappa;
-        const fix_t t = __double2ll_rn(hi * s);
-        return fix_store(t + __double2ll_rn((hi * s - (double)t) + lo * s));
-    };
     for (int k = 0; k < 36; ++k) {
         const double2 v = q[(size_t)k << g.lvb];
-        const int2 a = one(v.x), b = one(v.y);
+        const int2 a = fix_store(__double2ll_rn(v.x * s)), b = fix_store(__double2ll_rn(v.y * s));
         o[(size_t)k << g.lvb] = make_int4(a.x, a.y, b.x, b.y);
     }
 }
 
-int launch_fix_links(const Geom &g, const double2 *U64, int4 *out, int *d_bad, cudaStream_t s)
+int launch_fix_links(const Geom &g, const double2 *U64, double ks, int4 *out, int *d_bad, cudaStream_t s)
 {
-    k_fix_links<<<dim3(grid_for(g.V, 128), 4), 128, 0, s>>>(g, Gauge64{(double2 *)U64, g.lvb}, out, d_bad);
+    k_fix_links<<<dim3(grid_for(g.V, 128), 4), 128, 0, s>>>(g, Gauge64{(double2 *)U64, g.lvb}, ks, out, d_bad);
     MGC_CUDA(cudaGetLastError());
     count(1, (double)g.V * (2 * 576.0));
     return MGC_OK;
 }
 
-int launch_fix_clover(const Geom &g, const double2 *C64, double kappa, int4 *out, int *ex, int *d_bad, cudaStream_t s)
+int launch_fix_clover(const Geom &g, const double2 *C64, int ek, int4 *out, int2 *ex, int *d_bad, cudaStream_t s)
 {
-    k_fix_clover<<<grid_for(g.V, 128), 128, 0, s>>>(g, Clover64{(double2 *)C64, g.lvb}, kappa, out, ex, d_bad);
+    k_fix_clover<<<grid_for(g.V, 128), 128, 0, s>>>(g, Clover64{(double2 *)C64, g.lvb}, ek, out, ex, d_bad);
     MGC_CUDA(cudaGetLastError());
-    count(1, (double)g.V * (2 * 576.0 + 4.0));
+    count(1, (double)g.V * (2 * 576.0 + 8.0));
     return MGC_OK;
 }
 
-// D, D^dagger at FP64 in block fixed point (fix64.cuh).  24^3 x 48: 383 us
-// against 1259 us with FP64 instructions (2.7 TB/s of compulsory bytes against
+// D, D^dagger at FP64 in block fixed point (fix64.cuh).  24^3 x 48: 400 us
+// against 1259 us with FP64 instructions (2.5 TB/s of compulsory bytes against
 // 0.8); the FMA pipe's heavy half, where the widening products run, is busy 67 %
 // of the time.  Four blocks per SM (128 registers) and three (168) measure the
 // same; five spill (429 us).
@@ -290,7 +319,7 @@ __global__ void __launch_bounds__(FIX_THREADS, 4)
         for (int mu = 0; mu < 4; ++mu) g.lb[mu] = LVB / 4;
         src.lvb = dst.lvb = U.lvb = C.lvb = LVB;
     }
-    if (!fix_dirac_site<DAG>(g, i, src, dst, U, C, kappa, slots + threadIdx.x)) fix_fallback<DAG>(g, i, src, dst, Ud, Cd, kappa);
+    if (!fix_dirac_site<DAG>(g, i, src, dst, U, C, slots + threadIdx.x)) fix_fallback<DAG>(g, i, src, dst, Ud, Cd, kappa);
 }
 
 template <int LVB>
@@ -298,8 +327,8 @@ static void dirac_fix_launch(const mgc_clover_s *op, bool dag, Spinor64 in, Spin
 {
     const mgc_gauge_s *ga = op->gauge;
     const Geom &g = ga->lat->g;
-    const FixLinks U{ga->UQ, g.lvb};
-    const FixClover C{op->CQ, op->CE, g.lvb};
+    const FixLinks U{op->UQ, g.lvb};
+    const FixClover C{op->CQ, op->CE, op->fix_ek, g.lvb};
     const Gauge64 Ud{ga->U64, g.lvb};
     const Clover64 Cd{op->C64, g.lvb};
     dim3 grid(grid_for(g.V, FIX_THREADS), nrhs);

@@ -45,7 +45,7 @@ __global__ void __launch_bounds__(FIX_THREADS, 4) k_dirac_batch_fix(DiracBatchFi
         for (int mu = 0; mu < 4; ++mu) g.lb[mu] = LVB / 4;
         src.lvb = dst.lvb = U.lvb = C.lvb = LVB;
     }
-    if (!C.p || !fix_dirac_site<DAG>(g, i, src, dst, U, C, B.kappa[k], slots + threadIdx.x))
+    if (!C.p || !fix_dirac_site<DAG>(g, i, src, dst, U, C, slots + threadIdx.x))
         fix_fallback<DAG>(g, i, src, dst, B.U[k], B.C[k], B.kappa[k]);
 }
 
@@ -67,8 +67,8 @@ int dirac_batch_fix(const BatchSpec &spec, bool dag, const void *const *in, void
         B.end[k] = acc;
         B.in[k] = sp64(g, in[k]);
         B.out[k] = sp64(g, out[k]);
-        B.UQ[k] = FixLinks{op->gauge->UQ, g.lvb};
-        B.CQ[k] = FixClover{op->CQ, op->CE, g.lvb};
+        B.UQ[k] = FixLinks{op->UQ, g.lvb};
+        B.CQ[k] = FixClover{op->CQ, op->CE, op->fix_ek, g.lvb};
         B.U[k] = Gauge64{op->gauge->U64, g.lvb};
         B.C[k] = Clover64{op->C64, g.lvb};
         B.kappa[k] = op->kappa;

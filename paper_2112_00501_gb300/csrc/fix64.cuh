@@ -10,18 +10,21 @@
 // therefore takes three instructions of 1/16 the cost, which turns the operator
 // from one bound by the FP64 pipe into one bound by instruction issue and HBM.
 //
-// Scales.  Links are u = q 2^-60 (unitary to 1e-3, so |q| <= 2^60).  The clover
-// term is stored divided by kappa, q = (C/kappa) 2^(58 - e_C), e_C the site's
-// exponent (|C/kappa| < 2^e_C), so that D psi = kappa (C/kappa psi - H psi) needs
-// one multiplication per component.  A thread adds its eight hops and the
-// clover term in 64-bit integers in units of 2^(E - 56), E at least the
-// exponent of the largest component of psi at the nine sites: a neighbour's
-// components are brought to that unit as they are read (Q = psi 2^(60 - E)),
-// and where a neighbour exceeds E the sum is shifted down.  Sum bounds: a hop's
-// row has |sum| <= 4.9 (unitary rows, |h| <= 2 2^E), eight of them 2^5.3, the
-// clover term 2^5.46 (E >= e_psi + e_C - 2), together below 2^62.5 units; the
-// middle sums stay below 2^62.8 (two-norm bound for the links, eleven terms of
-// 2^57 + 2^59 for the clover).
+// Scales.  kappa = k' 2^ek with 1/2 <= |k'| < 1.  The links are stored times k',
+// q = k' u 2^60 (unitary to 1e-3, so |q| <= 2^60), the clover term as
+// q = C 2^(60 - e_C - ek), e_C the site's exponent (|C| < 2^(e_C + ek)).  A thread
+// adds its eight hops and the clover term in 64-bit integers in units of
+// 2^(E + ek - 56), E at least the exponent of the largest component of psi at the
+// nine sites: a neighbour's components are brought to that unit as they are read
+// (Q = psi 2^(60 - E)), and where a neighbour exceeds E the sum is shifted down.
+// The result is the sum times a power of two: one rounding.  Sum bounds: a hop's
+// row has |sum| <= 4.9 2^E (unitary rows, |h| <= 2 2^E), eight of them 2^5.3 2^E,
+// the clover term 2^5 2^E (E >= e_psi + room, a row's absolute sum of C below
+// 2^(5 + room + ek); room = 0 for kappa near 1/8), together below 2^62.2 units;
+// the middle sums stay below 2^62.9 (two-norm bound for the links; for the clover
+// eleven terms of 2^59 with its low limbs, and 2^31 times the row sum 2^30 of its
+// high limbs).  The dropped products a0 b0 are of random sign, 2^-57 of the
+// largest product in the mean square.
 //
 // A site is computed with FP64 instructions instead (fix_fallback) when its own
 // or a neighbour's components span more than 2^27, include some but not only
@@ -30,8 +33,12 @@
 // propagate, and no conversion needs a test of its own.  Gaussian components
 // fall below 2^-27 of their neighbourhood's largest once in 10^8.
 //
-// Error against 64 bits: each hop truncates at 2^(E - 56) (the -1/2 mean is
-// added back once), against FP64's rounding of every partial sum at 2^(E - 53).
+// Error against 64 bits: each hop is rounded at 2^(E + ek - 56), without bias (a
+// mean error of half a unit, the same everywhere, is a smooth field that the
+// solvers' low modes amplify), against FP64's rounding of every partial sum at
+// 2^(E - 53).  Against quadruple precision the operator is off by 6.3e-17 in the
+// 2-norm (kappa = 0.126 to 0.1365, c_SW = 1), with FP64 instructions by 1.7e-16;
+// the rounding of the exact result alone is 4.7e-17.
 #pragma once
 
 #include "hop.cuh"
@@ -44,8 +51,9 @@ typedef long long fix_t;
 constexpr int FIX_EMIN = 0x80;   // smallest biased exponent the fixed-point path takes
 constexpr int FIX_EMAX = 0x7c0;  // first biased exponent it does not
 
-// threads of a block, and the 16-byte staging slots each has in shared memory
-// (slot k of thread t at [k][t]): a neighbour's spinor and a link
+// threads of the operator's blocks, and the 16-byte staging slots a thread has in
+// shared memory (slot k of thread t at [k][t], NT threads): a neighbour's spinor
+// and a link
 constexpr int FIX_THREADS = 128;
 constexpr int FIX_SPINOR_SLOTS = 12, FIX_LINK_SLOTS = 9;
 
@@ -58,7 +66,7 @@ __device__ __forceinline__ void fix_copy16(int4 *dst, const void *src)
 __device__ __forceinline__ void fix_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N> __device__ __forceinline__ void fix_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
-// links: the plane order of Gauge64, a complex entry as (re hi, re lo, im hi, im lo)
+// links times k': the plane order of Gauge64, a complex entry as (re hi, re lo, im hi, im lo)
 struct FixLinks {
     const int4 *p;
     int lvb;
@@ -68,10 +76,11 @@ struct FixLinks {
     }
 };
 
-// C/kappa: the plane order of Clover64, and the exponent of every site
+// C: the plane order of Clover64, every site's (exponent, room), and ek
 struct FixClover {
     const int4 *p;
-    const int *e;
+    const int2 *e;
+    int ek;
     int lvb;
     __device__ __forceinline__ const int4 *at(int i) const
     {
@@ -121,11 +130,11 @@ struct FixRaw {
         for (int k = 0; k < 12; ++k) w[k] = __ldg(q + ((size_t)k << in.lvb));
     }
     // from the thread's staging slots
-    __device__ __forceinline__ void load_staged(const int4 *slot)
+    __device__ __forceinline__ void load_staged(const int4 *slot, int nt)
     {
 #pragma unroll
         for (int k = 0; k < 12; ++k) {
-            const int4 v = slot[k * FIX_THREADS];
+            const int4 v = slot[k * nt];
             w[k] = make_uint4(v.x, v.y, v.z, v.w);
         }
     }
@@ -187,7 +196,7 @@ __device__ __forceinline__ void fix_limbs(fix_t q, int &hi, int &lo)
     asm("" : "+r"(lo), "+r"(hi));  // 32-bit numbers of unknown origin (above)
 }
 
-// hh + mid 2^-32 in units of hh, rounded down
+// hh + mid 2^-32 in units of hh, rounded down (the sums start from half a unit)
 __device__ __forceinline__ fix_t fix_join(fix_t hh, fix_t mid) { return mac64((int)(mid >> 32), 1, hh); }
 
 // (a, b) + sgn P (l0, l1) with P the spin map of direction MU: the projected
@@ -230,31 +239,17 @@ __device__ __forceinline__ void fix_reconstruct(Cx<fix_t> &a, Cx<fix_t> &b, Cx<f
     default: CALL(3, +1); break;       \
     }
 
-// The projected half spinor of direction m (above) from the spinor in the
-// staging slots (negated where `flip`, conjugated where `back`), as limbs; raises E (and shifts acc down) where the neighbour
-// exceeds it; FIX_LEAVE when the site needs FP64.
-enum { FIX_LEAVE, FIX_ZERO, FIX_HOP };
-__device__ __forceinline__ int fix_half_spinor(const int4 *slot, int m, bool back, bool flip, Cx<fix_t> acc[12],
-                                                int &E, int h1[12], int h0[12])
+// The limbs of the half spinor projected for direction m (above) from the
+// components q(k) of a neighbour, conjugated for a backward hop; colour by
+// colour, so that few 64-bit intermediates live at a time
+template <class Q>
+__device__ __forceinline__ void fix_project_limbs(Q q, int m, bool back, int h1[12], int h0[12])
 {
-    FixRaw r;
-    r.load_staged(slot);
-    r.range();
-    if (r.emax > E) {
-        const int d = min(r.emax - E, 63);
-        E = r.emax;
-#pragma unroll
-        for (int k = 0; k < 12; ++k) acc[k] = Cx<fix_t>{acc[k].r >> d, acc[k].i >> d};
-    }
-    if (!fix_in_range(r, E)) return fix_all_zero(r) ? FIX_ZERO : FIX_LEAVE;
-    const int K = E + 4;
-    const uint32_t fm = flip ? ~0u : 0u;
     const fix_t bm = back ? -1 : 0;
-    // colour by colour, so that few 64-bit intermediates live at a time
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        Cx<fix_t> a = fix_component(r, k, K, fm), b = fix_component(r, 3 + k, K, fm);
-        const Cx<fix_t> l0 = fix_component(r, 6 + k, K, fm), l1 = fix_component(r, 9 + k, K, fm);
+        Cx<fix_t> a = q(k), b = q(3 + k);
+        const Cx<fix_t> l0 = q(6 + k), l1 = q(9 + k);
 #define MGC_FIX_CALL(MU, SGN) fix_project<MU, SGN>(a, b, l0, l1)
         MGC_FIX_SWITCH(m, MGC_FIX_CALL)
 #undef MGC_FIX_CALL
@@ -265,34 +260,60 @@ __device__ __forceinline__ int fix_half_spinor(const int4 *slot, int m, bool bac
         fix_limbs(b.r, h1[2 * k + 6], h0[2 * k + 6]);
         fix_limbs(b.i, h1[2 * k + 7], h0[2 * k + 7]);
     }
+}
+
+// The projected half spinor of direction m (above) from the spinor in the
+// staging slots (negated where `flip`, conjugated where `back`), as limbs; raises E (and shifts acc down) where the neighbour
+// exceeds it; FIX_LEAVE when the site needs FP64.
+enum { FIX_LEAVE, FIX_ZERO, FIX_HOP };
+__device__ __forceinline__ int fix_half_spinor(const int4 *slot, int nt, int m, bool back, bool flip, Cx<fix_t> acc[12],
+                                                int &E, int h1[12], int h0[12])
+{
+    FixRaw r;
+    r.load_staged(slot, nt);
+    r.range();
+    if (r.emax > E) {
+        const int d = min(r.emax - E, 62);
+        const fix_t half = (fix_t)1 << (d - 1);
+        E = r.emax;
+#pragma unroll
+        for (int k = 0; k < 12; ++k) acc[k] = Cx<fix_t>{(acc[k].r + half) >> d, (acc[k].i + half) >> d};
+    }
+    if (!fix_in_range(r, E)) return fix_all_zero(r) ? FIX_ZERO : FIX_LEAVE;
+    const int K = E + 4;
+    const uint32_t fm = flip ? ~0u : 0u;
+    fix_project_limbs([&](int k) { return fix_component(r, k, K, fm); }, m, back, h1, h0);
     return FIX_HOP;
 }
 
 // acc += the hop of direction m from its projected half spinor h (conjugated for
-// a backward hop) and the link in the staging slots.  U^dagger h is the conjugate
+// a backward hop) and the link whose entry k is at link[k stride] (shared or
+// global memory).  U^dagger h is the conjugate
 // of U^T conj(h): the backward hop reads the transposed entries and negates the
-// imaginary parts on the way in and out, as one's complements.
-__device__ __forceinline__ void fix_hop(const int4 *slot, int m, bool back, const int h1[12], const int h0[12],
-                                        Cx<fix_t> acc[12])
+// imaginary parts on the way in and out, as one's complements (~w = -w - 1, which
+// the rounding constant of the imaginary parts makes up for).
+__device__ __forceinline__ void fix_hop(const int4 *link, int stride, int m, bool back, const int h1[12],
+                                        const int h0[12], Cx<fix_t> acc[12])
 {
-    const int sa = (back ? 1 : 3) * FIX_THREADS, sb = (back ? 3 : 1) * FIX_THREADS;
+    const int sa = (back ? 1 : 3) * stride, sb = (back ? 3 : 1) * stride;
     const fix_t bm = back ? -1 : 0;
+    const fix_t cr = 0x80000000LL, ci = back ? -0x80000000LL : 0x80000000LL;  // half a unit of hh
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         fix_t hr[2], hi[2], mr[2], mi[2];
 #pragma unroll
         for (int b = 0; b < 3; ++b) {
-            const int4 u = slot[a * sa + b * sb];
+            const int4 u = link[a * sa + b * sb];
             const int n1 = fix_neg(u.z), n0 = fix_neg(u.w);
 #pragma unroll
             for (int s = 0; s < 2; ++s) {
                 const int k = 2 * (3 * s + b);
                 const int x1 = h1[k], x0 = h0[k], y1 = h1[k + 1], y0 = h0[k + 1];
                 hr[s] = mac64(n1, y1, b ? mac64(u.x, x1, hr[s]) : mul64(u.x, x1));
-                mr[s] = mac64(u.y, x1, b ? mac64(u.x, x0, mr[s]) : mul64(u.x, x0));
+                mr[s] = mac64(u.y, x1, mac64(u.x, x0, b ? mr[s] : cr));
                 mr[s] = mac64(n0, y1, mac64(n1, y0, mr[s]));
                 hi[s] = mac64(u.z, x1, b ? mac64(u.x, y1, hi[s]) : mul64(u.x, y1));
-                mi[s] = mac64(u.y, y1, b ? mac64(u.x, y0, mi[s]) : mul64(u.x, y0));
+                mi[s] = mac64(u.y, y1, mac64(u.x, y0, b ? mi[s] : ci));
                 mi[s] = mac64(u.w, x1, mac64(u.z, x0, mi[s]));
             }
         }
@@ -323,18 +344,20 @@ __device__ __forceinline__ int fix_neighbour(const Geom &g, const int c[4], int 
     return site_index(g, n);
 }
 
-// acc = C/kappa psi in the sum's unit: the products' unit times 2^L, L <= 4
-__device__ __forceinline__ void fix_clover(const FixClover &C, int i, const FixRaw &r, int K, int L,
-                                           Cx<fix_t> acc[12])
+// acc = C psi in the sum's unit, from psi's components q(k): the products'
+// unit times 2^L, L < 32
+template <class Q>
+__device__ __forceinline__ void fix_clover(const FixClover &C, int i, Q psi, int L, Cx<fix_t> acc[12])
 {
     const int4 *cp = C.at(i);
+    const fix_t half = 0x80000000LL >> max(L, 0);  // half a unit of the sum
 #pragma unroll
     for (int chi = 0; chi < 2; ++chi) {
         int v1[12], v0[12];
         fix_t hh[12], mid[12];
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
-            const Cx<fix_t> q = fix_component(r, 6 * chi + k, K);
+            const Cx<fix_t> q = psi(6 * chi + k);
             fix_limbs(q.r, v1[2 * k], v0[2 * k]);
             fix_limbs(q.i, v1[2 * k + 1], v0[2 * k + 1]);
         }
@@ -344,9 +367,9 @@ __device__ __forceinline__ void fix_clover(const FixClover &C, int i, const FixR
 #pragma unroll
             for (int z = 0; z < 2; ++z) {
                 hh[4 * k + z] = mul64(d.x, v1[4 * k + z]);
-                mid[4 * k + z] = mac64(d.x, v0[4 * k + z], mul64(d.y, v1[4 * k + z]));
+                mid[4 * k + z] = mac64(d.x, v0[4 * k + z], mac64(d.y, v1[4 * k + z], half));
                 hh[4 * k + 2 + z] = mul64(d.z, v1[4 * k + 2 + z]);
-                mid[4 * k + 2 + z] = mac64(d.z, v0[4 * k + 2 + z], mul64(d.w, v1[4 * k + 2 + z]));
+                mid[4 * k + 2 + z] = mac64(d.z, v0[4 * k + 2 + z], mac64(d.w, v1[4 * k + 2 + z], half));
             }
         }
         int k = 3;
@@ -380,7 +403,7 @@ __device__ __forceinline__ void fix_clover(const FixClover &C, int i, const FixR
         for (int m = 0; m < 12; ++m) {
             const fix_t y = fix_join(hh[m], mid[m]);
             fix_t r;
-            if (L >= 0) {  // up to four bits of the middle sum below hh's unit
+            if (L >= 0) {  // bits of the middle sum below hh's unit
                 const uint32_t lo = __funnelshift_l((uint32_t)mid[m], (uint32_t)y, L);
                 const uint32_t hi = __funnelshift_l((uint32_t)y, (uint32_t)(y >> 32), L);
                 r = (fix_t)(((unsigned long long)hi << 32) | lo);
@@ -405,26 +428,27 @@ __device__ __noinline__ void fix_fallback(const Geom &g, int i, const Spinor64 &
     out.store(i, o[0]);
 }
 
-// out(i) = (D psi)(i) in fixed point; false (nothing stored) when the site needs
-// FP64.  `slots` is the thread's column of the block's staging slots.  One copy
-// of the hop's code serves all eight: unrolled per direction the kernel is 12,600
-// instructions long and waits on instruction fetch for half its time (1060 us on
-// 24^3 x 48).  The next hop's spinor and link are copied to shared memory while
-// this hop's products run; without that, loads were the first stall (433 us).
+// (D psi)(i) = -2^(E + ek - 1078) acc in fixed point (E the biased exponent);
+// false when the site needs FP64.  `slots` is the thread's column of the block's
+// staging slots, nt its threads.  One copy of the hop's code serves all eight:
+// unrolled per direction the kernel is 12,600 instructions long and waits on
+// instruction fetch for half its time (1060 us on 24^3 x 48).  The next hop's
+// spinor and link are copied to shared memory while this hop's products run;
+// without that, loads were the first stall (433 us).
 template <bool DAG>
-__device__ __forceinline__ bool fix_dirac_site(const Geom &g, int i, const Spinor64 &in, const Spinor64 &out,
-                                               const FixLinks &U, const FixClover &C, double kappa, int4 *slots)
+__device__ __forceinline__ bool fix_dirac_sum(const Geom &g, int i, const Spinor64 &in, const FixLinks &U,
+                                              const FixClover &C, int4 *slots, int nt, Cx<fix_t> acc[12], int &E)
 {
-    int4 *const ls = slots + FIX_SPINOR_SLOTS * FIX_THREADS;
+    int4 *const ls = slots + FIX_SPINOR_SLOTS * nt;
     auto copy_spinor = [&](int j) {
         const double2 *q = in.at(j);
 #pragma unroll
-        for (int k = 0; k < FIX_SPINOR_SLOTS; ++k) fix_copy16(slots + k * FIX_THREADS, q + ((size_t)k << in.lvb));
+        for (int k = 0; k < FIX_SPINOR_SLOTS; ++k) fix_copy16(slots + k * nt, q + ((size_t)k << in.lvb));
     };
     auto copy_link = [&](int d, int j) {
         const int4 *q = U.at(d & 1 ? j : i, d >> 1);
 #pragma unroll
-        for (int k = 0; k < FIX_LINK_SLOTS; ++k) fix_copy16(ls + k * FIX_THREADS, q + ((size_t)k << U.lvb));
+        for (int k = 0; k < FIX_LINK_SLOTS; ++k) fix_copy16(ls + k * nt, q + ((size_t)k << U.lvb));
     };
     int c[4];
     site_coords(g, i, c);
@@ -435,34 +459,31 @@ __device__ __forceinline__ bool fix_dirac_site(const Geom &g, int i, const Spino
     copy_link(0, j);
     fix_commit();
 
-    Cx<fix_t> acc[12];
-    int E;
-    int state = FIX_HOP, zeros = 0;
+    int state = FIX_HOP;
     {
         FixRaw r;
         r.load(in, i);
         r.range();
-        const int eC = __ldg(C.e + i);
+        const int2 eC = __ldg(C.e + i);
         const int ep = max(r.emax, FIX_EMIN);
-        E = ep + max(0, eC - 2);
+        E = ep + eC.y;
         if (fix_in_range(r, ep)) {
-            fix_clover(C, i, r, ep + 4, eC + 2 + ep - E, acc);
+            fix_clover(C, i, [&](int k) { return fix_component(r, k, ep + 4); }, eC.x - eC.y, acc);
         } else {
             state = fix_all_zero(r) ? FIX_ZERO : FIX_LEAVE;
 #pragma unroll
             for (int k = 0; k < 12; ++k) acc[k] = Cx<fix_t>{0, 0};
         }
     }
-    // H enters with a minus sign: sum H - C/kappa, and -kappa at the end.  The
-    // eight hops' truncation is half a unit each on average.
+    // the sum is that of kappa H psi - C psi
 #pragma unroll
-    for (int k = 0; k < 12; ++k) acc[k] = Cx<fix_t>{4 - acc[k].r, 4 - acc[k].i};
+    for (int k = 0; k < 12; ++k) acc[k] = -acc[k];
 #pragma unroll 1
     for (int d = 0; d < 8 && state != FIX_LEAVE; ++d) {
         const int m = (d & ~1) + (int)((bool)(d & 1) != DAG);
         int h1[12], h0[12];
         fix_wait<1>();  // this hop's spinor (its link may be in flight)
-        state = fix_half_spinor(slots, m, d & 1, flip, acc, E, h1, h0);
+        state = fix_half_spinor(slots, nt, m, d & 1, flip, acc, E, h1, h0);
         if (d < 7) {
             // every slot has been read: the test above depends on all of them
             j = fix_neighbour(g, c, d + 1, flip);
@@ -470,18 +491,27 @@ __device__ __forceinline__ bool fix_dirac_site(const Geom &g, int i, const Spino
         }
         fix_commit();
         fix_wait<1>();  // this hop's link
-        if (state == FIX_HOP) fix_hop(ls, m, d & 1, h1, h0, acc);
-        else ++zeros;
+        if (state == FIX_HOP) fix_hop(ls, nt, m, d & 1, h1, h0, acc);
         if (d < 7) copy_link(d + 1, j);
         fix_commit();
     }
     fix_wait<0>();
     if (state == FIX_LEAVE) return false;
-    if (zeros) {  // their half units; nine zero sites give an exact zero
-#pragma unroll
-        for (int k = 0; k < 12; ++k) acc[k] = Cx<fix_t>{acc[k].r - (zeros >> 1), acc[k].i - (zeros >> 1)};
-    }
-    const double sc = -kappa * __hiloint2double((E - 55) << 20, 0);
+    return true;
+}
+
+// 2^(e - 1023) for a biased exponent 0 < e < 2047
+__device__ __forceinline__ double fix_pow2(int e) { return __hiloint2double(e << 20, 0); }
+
+// out(i) = (D psi)(i); false (nothing stored) when the site needs FP64
+template <bool DAG>
+__device__ __forceinline__ bool fix_dirac_site(const Geom &g, int i, const Spinor64 &in, const Spinor64 &out,
+                                               const FixLinks &U, const FixClover &C, int4 *slots)
+{
+    Cx<fix_t> acc[12];
+    int E;
+    if (!fix_dirac_sum<DAG>(g, i, in, U, C, slots, FIX_THREADS, acc, E)) return false;
+    const double sc = -fix_pow2(E + C.ek - 55);
     Cx<double> o[12];
 #pragma unroll
     for (int k = 0; k < 12; ++k)

@@ -21,7 +21,6 @@ struct mgc_lattice_s {
 struct mgc_gauge_s {
     mgc_lattice_s *lat;
     double2 *U64;  // packed FP64, 18 reals per link
-    int4 *UQ;      // the links in fixed point for the FP64 operator (NULL unless near unitary)
     void *U32;     // packed FP32 at compress (NULL when prec == 64)
     void *U16;     // packed FP16 at compress (NULL unless prec == 16)
     int prec;      // storage precision: 64, 32 or 16
@@ -37,8 +36,13 @@ struct mgc_clover_s {
     double kappa, csw;
     double2 *C64;   // packed FP64 clover C
     double2 *Ci64;  // packed FP64 C^-1
-    int4 *CQ;       // C/kappa in fixed point and its site exponents (NULL: D runs on FP64 units)
-    int *CE;
+    // fixed-point copies for the FP64 operator (CQ NULL: it runs on FP64 units):
+    // links times kappa 2^-fix_ek, C, and C's site exponents and rooms
+    int4 *UQ;
+    int4 *CQ;
+    int2 *CE;
+    int fix_ek;
+    int fix_room;  // the largest room
     void *C32;      // packed FP32 C (NULL when prec == 64)
     void *C16;      // packed FP16 C followed by its per-site scales (prec == 16)
     float *C16_sc;
@@ -100,9 +104,10 @@ int launch_pack(const Geom &g, int prec, int nrhs, const double *canon, void *pa
 int launch_unpack(const Geom &g, int prec, int nrhs, const void *packed, double *canon, cudaStream_t s);
 int launch_convert(const Geom &g, int nrhs, int pin, const void *in, int pout, void *out, cudaStream_t s);
 int launch_gauge_pack(const Geom &g, const double *canon_dev, int prec, int compress, void *out, cudaStream_t s);
-// fixed-point copies of the links and of C/kappa; *d_bad is set when a field is out of their range
-int launch_fix_links(const Geom &g, const double2 *U64, int4 *out, int *d_bad, cudaStream_t s);
-int launch_fix_clover(const Geom &g, const double2 *C64, double kappa, int4 *out, int *ex, int *d_bad, cudaStream_t s);
+// the links times ks, and C with the hopping's exponent ek, in fixed point (fix64.cuh);
+// d_bad[0] is set when a field is out of their range, d_bad[1] receives the largest room
+int launch_fix_links(const Geom &g, const double2 *U64, double ks, int4 *out, int *d_bad, cudaStream_t s);
+int launch_fix_clover(const Geom &g, const double2 *C64, int ek, int4 *out, int2 *ex, int *d_bad, cudaStream_t s);
 int launch_dirac(const mgc_clover_s *op, int prec, bool dag, const void *in, void *out, int nrhs,
                  cudaStream_t s);
 // w = D z with the FP32 operator for an FP16 z (FP32 result)

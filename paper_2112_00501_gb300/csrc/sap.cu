@@ -26,6 +26,7 @@
 // the odd sites apply C_oo^-1 (read from global memory) in between and finally
 // form e_o = C_oo^-1 (r_o + kappa H_oe e_e).  Odd entries of the shared vector
 // hold the odd-site intermediate, even entries the even-site residual.
+#include "fix64.cuh"
 #include "hop.cuh"
 #include "hop16.cuh"
 #include "mgc_host.h"
@@ -124,6 +125,44 @@ __device__ __forceinline__ void block_hop_dir(const GA &U, int blkbase, int i, i
         U.load(blkbase + nb, MU, u);
         su3_dag_mul(u, h, w);
         reconstruct_add<MU, +1>(acc, w);
+    }
+}
+
+// e += MR_nmr(D_B, rv), rv its domain residual (in shared memory rs as well)
+template <class GA, class CL, typename T>
+__device__ __forceinline__ void mr_domain(const GA &U, const CL &C, T kappa, int blkbase, int i, int l, int vb,
+                                          const int nf[4], const int nb[4], Cx<T> *rs, T *red, int nmr, Cx<T> rv[12],
+                                          Cx<T> e[12])
+{
+    for (int it = 0; it < nmr; ++it) {
+        Cx<T> acc[12];
+#pragma unroll
+        for (int k = 0; k < 12; ++k) acc[k] = Cx<T>{0, 0};
+        block_hop_dir<0>(U, blkbase, i, nf[0], nb[0], rs, vb, acc);
+        block_hop_dir<1>(U, blkbase, i, nf[1], nb[1], rs, vb, acc);
+        block_hop_dir<2>(U, blkbase, i, nf[2], nb[2], rs, vb, acc);
+        block_hop_dir<3>(U, blkbase, i, nf[3], nb[3], rs, vb, acc);
+        T cl[72];
+        C.load(i, cl);
+        Cx<T> p[12];
+        clover_mul(cl, rv, p);
+        T pr = 0, pi = 0, pp = 0;
+#pragma unroll
+        for (int k = 0; k < 12; ++k) {
+            p[k] = Cx<T>{fma(-kappa, acc[k].r, p[k].r), fma(-kappa, acc[k].i, p[k].i)};
+            pr = fma(p[k].r, rv[k].r, fma(p[k].i, rv[k].i, pr));
+            pi = fma(p[k].r, rv[k].i, fma(-p[k].i, rv[k].r, pi));
+            pp = fma(p[k].r, p[k].r, fma(p[k].i, p[k].i, pp));
+        }
+        block_sum3(pr, pi, pp, red);
+        const Cx<T> alpha = (pp > 0) ? Cx<T>{pr / pp, pi / pp} : Cx<T>{0, 0};
+#pragma unroll
+        for (int k = 0; k < 12; ++k) {
+            e[k] = cfma(alpha, rv[k], e[k]);
+            rv[k] = rv[k] - alpha * p[k];
+            rs[k * vb + l] = rv[k];
+        }
+        __syncthreads();
     }
 }
 
@@ -303,40 +342,310 @@ __global__ void __launch_bounds__(256) k_sap_colour(Geom g, SP b, SP x, GA U, CL
     }
 
     // 2. minimal residual on D_B
-    for (int it = 0; it < nmr; ++it) {
-        Cx<T> acc[12];
-#pragma unroll
-        for (int k = 0; k < 12; ++k) acc[k] = Cx<T>{0, 0};
-        block_hop_dir<0>(U, blkbase, i, nf[0], nb[0], rs, vb, acc);
-        block_hop_dir<1>(U, blkbase, i, nf[1], nb[1], rs, vb, acc);
-        block_hop_dir<2>(U, blkbase, i, nf[2], nb[2], rs, vb, acc);
-        block_hop_dir<3>(U, blkbase, i, nf[3], nb[3], rs, vb, acc);
-        T cl[72];
-        C.load(i, cl);
-        Cx<T> p[12];
-        clover_mul(cl, rv, p);
-        T pr = 0, pi = 0, pp = 0;
-#pragma unroll
-        for (int k = 0; k < 12; ++k) {
-            p[k] = Cx<T>{fma(-kappa, acc[k].r, p[k].r), fma(-kappa, acc[k].i, p[k].i)};
-            pr = fma(p[k].r, rv[k].r, fma(p[k].i, rv[k].i, pr));
-            pi = fma(p[k].r, rv[k].i, fma(-p[k].i, rv[k].r, pi));
-            pp = fma(p[k].r, p[k].r, fma(p[k].i, p[k].i, pp));
-        }
-        block_sum3(pr, pi, pp, red);
-        const Cx<T> alpha = (pp > 0) ? Cx<T>{pr / pp, pi / pp} : Cx<T>{0, 0};
-#pragma unroll
-        for (int k = 0; k < 12; ++k) {
-            e[k] = cfma(alpha, rv[k], e[k]);
-            rv[k] = rv[k] - alpha * p[k];
-            rs[k * vb + l] = rv[k];
-        }
-        __syncthreads();
-    }
+    mr_domain(U, C, kappa, blkbase, i, l, vb, nf, nb, rs, red, nmr, rv, e);
 
     // 3. x_B += e
     if (!x_zero) {
         Cx<T> xo[12];
+        xx.load(i, xo);
+#pragma unroll
+        for (int k = 0; k < 12; ++k) e[k] = e[k] + xo[k];
+    }
+    xx.store(i, e);
+}
+
+// ------------------------------------------------------------------ FP64 MR in fixed point
+// The FP64 smoother with MR domain solves in block fixed point (fix64.cuh): the
+// domain residual by the fixed-point operator, and D_B r with r kept in shared
+// memory as 64-bit integers in one unit for the whole domain,
+// r = Q 2^(E - 1082) with |Q| < 2^(60 - dE), E (biased) from the domain's largest
+// component and dE the room the lattice's clover terms take (fix64.cuh), and
+// D_B r = -2^(E + ek - 1078) acc.  The inner products, alpha, e and r - alpha p
+// are FP64 as before, on the integers' doubles r' and p': with
+// beta = <p', r'>/<p', p'>, alpha = -beta 2^(-4 - ek) and r - alpha p is
+// 2^(E - 1082) (r' - beta p').  A domain whose residual is not finite or outside
+// 2^-894 .. 2^961 runs on FP64 instructions (mr_domain_fp64).
+//
+// Bound: FP64 pipe (56 % busy; conversions, inner products and updates) and the
+// widening products in turn.  r and e in shared memory (98 KB) and 128 registers
+// give two blocks per SM; the residual's staging slots lie over r and e, which
+// come later.  16^3 x 32, 4 steps: 281 us a colour against 883 us with FP64
+// instructions.  Error of two sweeps against quadruple precision on 8^4: 1.0e-16
+// against 2.3e-16.
+
+// Q of a double, K = the unit's biased exponent + 4: x = Q 2^(K - 1086) rounded
+// towards zero, |x| < 2^(K - 1026)
+__device__ __forceinline__ fix_t fix_from_any(double x, int K)
+{
+    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+    const int e = (int)(hi >> 20) & 0x7ff;
+    const int s = K - e;
+    unsigned long long m = ((unsigned long long)(__funnelshift_l(lo, hi, 11) | 0x80000000u) << 32) | (lo << 11);
+    m = (e == 0 || s > 63) ? 0 : m >> s;
+    return (int)hi < 0 ? -(fix_t)m : (fix_t)m;
+}
+
+// the largest biased exponent of 24 reals
+__device__ __forceinline__ int fix_exponent(const Cx<double> v[12])
+{
+    float mx = 0.f;
+#pragma unroll
+    for (int k = 0; k < 12; ++k)
+        mx = max3abs(mx, __int_as_float(__double2hiint(v[k].r)), __int_as_float(__double2hiint(v[k].i)));
+    return __float_as_int(mx) >> 20;
+}
+
+// the block's maximum of a non-negative integer, the same on every thread
+__device__ __forceinline__ int block_max(int v, int *red)
+{
+    const int nt = blockDim.x;
+    v = __reduce_max_sync(nt >= 32 ? 0xffffffffu : (1u << nt) - 1u, v);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+    __syncthreads();
+    v = 0;
+    for (int w = 0; w < ((nt + 31) >> 5); ++w) v = max(v, red[w]);
+    return v;
+}
+
+// s + t and its rounding error
+__device__ __forceinline__ double two_sum(double s, double t, double &err)
+{
+    const double r = s + t, b = r - s;
+    err = (s - (r - b)) + (t - b);
+    return r;
+}
+
+// alpha = (pr + i pi)/pp of the block's sums: block_sum3 with the warps' partials
+// added pairwise in double-double by the lanes of each warp, and quotients with
+// their remainders, so that alpha's error (which every component of e shares) is
+// little more than its own rounding.  A zero pp gives zero.
+__device__ __forceinline__ Cx<double> block_alpha(double pr, double pi, double pp, double *red)
+{
+    const int nt = blockDim.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const unsigned mask = nt >= 32 ? 0xffffffffu : ((1u << nt) - 1u);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+        if (o < nt) {
+            pr += __shfl_xor_sync(mask, pr, o);
+            pi += __shfl_xor_sync(mask, pi, o);
+            pp += __shfl_xor_sync(mask, pp, o);
+        }
+    double prl = 0, pil = 0, ppl = 0;
+    if (nt > 32) {
+        if (lane < 3) red[(lane << 3) + warp] = lane == 0 ? pr : (lane == 1 ? pi : pp);
+        __syncthreads();
+        // lane 8 v + w holds warp w's partial of value v (at most eight warps)
+        double s = lane < 24 && (lane & 7) < (nt >> 5) ? red[lane] : 0.0, lo = 0;
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1) {
+            double err;
+            const double t = __shfl_xor_sync(mask, s, o), tl = __shfl_xor_sync(mask, lo, o);
+            s = two_sum(s, t, err);
+            lo = (lo + tl) + err;
+        }
+        pr = __shfl_sync(mask, s, 0);
+        pi = __shfl_sync(mask, s, 8);
+        pp = __shfl_sync(mask, s, 16);
+        prl = __shfl_sync(mask, lo, 0);
+        pil = __shfl_sync(mask, lo, 8);
+        ppl = __shfl_sync(mask, lo, 16);
+    } else {
+        __syncthreads();
+    }
+    if (!(pp > 0)) return Cx<double>{0, 0};
+    const double inv = 1.0 / pp;
+    const double qr = pr * inv, qi = pi * inv;
+    return Cx<double>{fma(fma(-qr, pp, pr) + fma(-qr, ppl, prl), inv, qr),
+                      fma(fma(-qi, pp, pi) + fma(-qi, ppl, pil), inv, qi)};
+}
+
+__device__ __noinline__ void mr_domain_fp64(const Gauge64 &U, const Clover64 &C, double kappa, int blkbase, int i,
+                                            int l, int vb, const Geom &g, const int *lc, Cx<double> *rs, double *red,
+                                            int nmr, Cx<double> *rv, Cx<double> *e)
+{
+    int nf[4], nb[4];
+#pragma unroll
+    for (int mu = 0; mu < 4; ++mu) {
+        int t[4] = {lc[0], lc[1], lc[2], lc[3]};
+        t[mu] = lc[mu] + 1;
+        nf[mu] = (t[mu] < (1 << g.lb[mu])) ? local_index(g, t) : -1;
+        t[mu] = lc[mu] - 1;
+        nb[mu] = (t[mu] >= 0) ? local_index(g, t) : -1;
+    }
+#pragma unroll
+    for (int k = 0; k < 12; ++k) rs[k * vb + l] = rv[k];
+    __syncthreads();
+    mr_domain(U, C, kappa, blkbase, i, l, vb, nf, nb, rs, red, nmr, rv, e);
+}
+
+__device__ __noinline__ void dirac_site_fp64(const Geom &g, int i, const Spinor64 &x, const Gauge64 &U,
+                                             const Clover64 &C, double kappa, Cx<double> *out)
+{
+    int c[4];
+    site_coords(g, i, c);
+    dirac_site<false>(g, c, i, x, U, C, kappa, out);
+}
+
+constexpr size_t sap_fix_smem(int vb) { return (size_t)vb * 24 * 16 + 96 * sizeof(double) + 32 * sizeof(int); }
+
+template <int LVB>
+__global__ void __launch_bounds__(256, 2) k_sap_fix(Geom g, Spinor64 b, Spinor64 x, FixLinks U, FixClover C, Gauge64 Ud,
+                                                    Clover64 Cd, double kappa, int dE, int colour, int nmr, int x_zero)
+{
+    extern __shared__ __align__(128) unsigned char smem[];
+    if (LVB > 0) {
+        g.lvb = LVB;
+#pragma unroll
+        for (int mu = 0; mu < 4; ++mu) g.lb[mu] = LVB / 4;
+        b.lvb = x.lvb = U.lvb = C.lvb = LVB;
+    }
+    const int vb = 1 << g.lvb;
+    longlong2 *const rs = reinterpret_cast<longlong2 *>(smem);
+    double2 *const es = reinterpret_cast<double2 *>(rs + 12 * vb);
+    double *const red = reinterpret_cast<double *>(es + 12 * vb);
+    int *const redi = reinterpret_cast<int *>(red + 96);
+
+    const int l = threadIdx.x;
+    const Spinor64 bb = shift_rhs(b, blockIdx.y, g.V), xx = shift_rhs(x, blockIdx.y, g.V);
+    int j = blockIdx.x;
+    const int half0 = g.NB[0] >> 1;
+    int bc[4], lc[4];
+    const int m0 = j % half0;
+    j /= half0;
+    bc[1] = j % g.NB[1];
+    j /= g.NB[1];
+    bc[2] = j % g.NB[2];
+    bc[3] = j / g.NB[2];
+    bc[0] = 2 * m0 + ((colour + bc[1] + bc[2] + bc[3]) & 1);
+    const int blkbase = block_index(g, bc) << g.lvb;
+    const int i = blkbase | l;
+    local_coords(g, l, lc);
+
+    // 1. block residual
+    Cx<double> rv[12];
+    if (!x_zero) {
+        Cx<fix_t> acc[12];
+        int E;
+        if (fix_dirac_sum<false>(g, i, xx, U, C, reinterpret_cast<int4 *>(smem) + l, vb, acc, E)) {
+            const double sc = fix_pow2(E + C.ek - 55);
+            bb.load(i, rv);
+#pragma unroll
+            for (int k = 0; k < 12; ++k)
+                rv[k] = Cx<double>{fma(sc, __ll2double_rn(acc[k].r), rv[k].r),
+                                   fma(sc, __ll2double_rn(acc[k].i), rv[k].i)};
+        } else {
+            Cx<double> dx[12];
+            dirac_site_fp64(g, i, xx, Ud, Cd, kappa, dx);
+            bb.load(i, rv);
+#pragma unroll
+            for (int k = 0; k < 12; ++k) rv[k] = rv[k] - dx[k];
+        }
+    } else {
+        bb.load(i, rv);
+    }
+    const int e0 = block_max(fix_exponent(rv), redi);  // a barrier: the staging slots are free
+    if (e0 >= FIX_EMAX || (e0 < FIX_EMIN && e0 > 0)) {
+        Cx<double> r[12], e[12];
+#pragma unroll
+        for (int k = 0; k < 12; ++k) {
+            r[k] = rv[k];
+            e[k] = Cx<double>{0, 0};
+        }
+        mr_domain_fp64(Ud, Cd, kappa, blkbase, i, l, vb, g, lc, reinterpret_cast<Cx<double> *>(smem), red, nmr, r, e);
+        if (!x_zero) {
+            Cx<double> xo[12];
+            xx.load(i, xo);
+#pragma unroll
+            for (int k = 0; k < 12; ++k) e[k] = e[k] + xo[k];
+        }
+        xx.store(i, e);
+        return;
+    }
+
+    // 2. minimal residual
+#pragma unroll
+    for (int k = 0; k < 12; ++k) es[k * vb + l] = make_double2(0.0, 0.0);
+    const int2 eC = __ldg(C.e + i);
+    int E = e0 + dE, K = e0 + dE + 4;
+#pragma unroll 1
+    for (int it = 0; it < nmr && E > FIX_EMIN / 2 + 32 + dE; ++it) {
+        // r in the domain's unit (a zero residual has e0 = 0 and no step)
+#pragma unroll
+        for (int k = 0; k < 12; ++k)
+            rs[k * vb + l] = make_longlong2(fix_from_any(rv[k].r, K), fix_from_any(rv[k].i, K));
+        __syncthreads();
+        Cx<fix_t> acc[12];
+        fix_clover(C, i,
+                   [&](int k) {
+                       const longlong2 v = rs[k * vb + l];
+                       return Cx<fix_t>{v.x, v.y};
+                   },
+                   eC.x, acc);
+#pragma unroll
+        for (int k = 0; k < 12; ++k) acc[k] = -acc[k];
+#pragma unroll 1
+        for (int d = 0; d < 8; ++d) {
+            const int mu = d >> 1;
+            const bool back = d & 1;
+            int n[4];
+            bool in = true;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                n[k] = lc[k] + (k == mu ? (back ? -1 : 1) : 0);
+                in = in && n[k] >= 0 && n[k] < (1 << g.lb[k]);
+            }
+            if (in) {
+                const int ln = local_index(g, n);
+                int h1[12], h0[12];
+                fix_project_limbs(
+                    [&](int k) {
+                        const longlong2 v = rs[k * vb + ln];
+                        return Cx<fix_t>{v.x, v.y};
+                    },
+                    d, back, h1, h0);
+                fix_hop(U.at(back ? blkbase | ln : i, mu), vb, d, back, h1, h0, acc);
+            }
+        }
+        // inner products of p' and r' (the integers as doubles), then r' - beta p'
+        double pr = 0, pi = 0, pp = 0;
+        Cx<double> p[12];
+#pragma unroll
+        for (int k = 0; k < 12; ++k) {
+            const longlong2 v = rs[k * vb + l];
+            const double rr = __ll2double_rn(v.x), ri = __ll2double_rn(v.y);
+            p[k] = Cx<double>{__ll2double_rn(acc[k].r), __ll2double_rn(acc[k].i)};
+            pr = fma(p[k].r, rr, fma(p[k].i, ri, pr));
+            pi = fma(p[k].r, ri, fma(-p[k].i, rr, pi));
+            pp = fma(p[k].r, p[k].r, fma(p[k].i, p[k].i, pp));
+        }
+        const Cx<double> beta = block_alpha(pr, pi, pp, red);
+        const Cx<double> a = -fix_pow2(E - 63 - C.ek) * beta;  // r = 2^(E - 1082) r', alpha = -beta 2^(-4 - ek)
+#pragma unroll
+        for (int k = 0; k < 12; ++k) {
+            const longlong2 v = rs[k * vb + l];
+            const Cx<double> r = {__ll2double_rn(v.x), __ll2double_rn(v.y)};
+            const double2 e = es[k * vb + l];
+            const Cx<double> en = cfma(a, r, Cx<double>{e.x, e.y});
+            es[k * vb + l] = make_double2(en.r, en.i);
+            rv[k] = r - beta * p[k];
+        }
+        if (it + 1 < nmr) {
+            // rv is in units of 2^(E - 1082); a zero residual ends the loop
+            const int e1 = block_max(fix_exponent(rv), redi);
+            K = e1 + dE + 4;
+            E = e1 == 0 ? 0 : e1 + E - 1082 + dE;
+        }
+    }
+
+    // 3. x_B += e
+    Cx<double> e[12];
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+        const double2 v = es[k * vb + l];
+        e[k] = Cx<double>{v.x, v.y};
+    }
+    if (!x_zero) {
+        Cx<double> xo[12];
         xx.load(i, xo);
 #pragma unroll
         for (int k = 0; k < 12; ++k) e[k] = e[k] + xo[k];
@@ -1979,6 +2288,33 @@ static int sap_run(const Geom &g, SP b, SP x, GA U, CL C, CL Ci, double kappa, i
     return MGC_OK;
 }
 
+// The largest room the fixed-point MR leaves for the clover term: beyond it
+// (kappa below about 1/1000) r would keep less than FP64's 53 bits below the
+// domain's largest component.
+constexpr int SAP_FIX_MAX_ROOM = 6;
+
+template <int LVB>
+static int sap_run_fix(const mgc_clover_s *op, const void *b, void *x, int nrhs, int n_cy, int n_mr, int x_is_zero,
+                       cudaStream_t s)
+{
+    const Geom &g = op->gauge->lat->g;
+    const int vb = 1 << g.lvb;
+    const size_t smem = sap_fix_smem(vb);
+    MGC_CUDA(cudaFuncSetAttribute(k_sap_fix<LVB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    dim3 grid(g.nblocks / 2, nrhs);
+    for (int cy = 0; cy < n_cy; ++cy)
+        for (int colour = 0; colour < 2; ++colour) {
+            const int xz = (cy == 0 && colour == 0) ? x_is_zero : 0;
+            k_sap_fix<LVB><<<grid, vb, smem, s>>>(
+                g, Spinor64{(double2 *)b, g.lvb}, Spinor64{(double2 *)x, g.lvb}, FixLinks{op->UQ, g.lvb},
+                FixClover{op->CQ, op->CE, op->fix_ek, g.lvb}, Gauge64{op->gauge->U64, g.lvb}, Clover64{op->C64, g.lvb}, op->kappa,
+                op->fix_room, colour, n_mr, xz);
+            count(1, sap_launch_bytes(g, 64, 18, nrhs, xz != 0));
+        }
+    MGC_CUDA(cudaGetLastError());
+    return MGC_OK;
+}
+
 // the smoother: MR on D_B (clover C), Jacobi on A_B (clover C^-1) or even-odd
 // MR on D_B (clover C, odd-site C^-1 from global memory)
 template <int MODE>
@@ -1990,6 +2326,11 @@ static int sap_launch_impl(const mgc_clover_s *op, int prec, const void *b, void
     constexpr bool jac = MODE == SAP_JAC;
     if ((1 << g.lvb) > 256) return fail(MGC_ERR_UNSUPPORTED_SHAPE, "SAP domains are limited to 256 sites");
     if (prec == 64) {
+        if (MODE == SAP_MR && op->CQ && op->fix_room <= SAP_FIX_MAX_ROOM) {
+            const bool cube = g.lb[0] == g.lb[1] && g.lb[1] == g.lb[2] && g.lb[2] == g.lb[3];
+            return cube && g.lvb == 8 ? sap_run_fix<8>(op, b, x, nrhs, n_cy, n_it, x_is_zero, s)
+                                      : sap_run_fix<0>(op, b, x, nrhs, n_cy, n_it, x_is_zero, s);
+        }
         return sap_run<MODE>(g, Spinor64{(double2 *)b, g.lvb}, Spinor64{(double2 *)x, g.lvb}, Gauge64{ga->U64, g.lvb},
                              Clover64{jac ? op->Ci64 : op->C64, g.lvb}, Clover64{op->Ci64, g.lvb}, op->kappa, nrhs,
                              n_cy, n_it, x_is_zero, s, prec, ga->compress);

@@ -42,7 +42,7 @@ def _check(name, psi, tol=6e-16, U=None, kappa=None, dagger=False, p=0):
 
 @pytest.mark.parametrize("name", ["c0_4^4", "ragged_8x4x12x8", "mid_8^4"])
 @pytest.mark.parametrize("dagger", [False, True])
-@pytest.mark.parametrize("kappa", [0.01, 0.13, -0.13, 0.8, 70.0])  # 0.01 and 70 run on FP64 instructions
+@pytest.mark.parametrize("kappa", [0.0, 1e-6, 0.01, 0.13, -0.13, 0.8, 70.0])  # 0 and 1e-6 run on FP64 instructions
 def test_error(name, dagger, kappa):
     _check(name, fields(name)[6], kappa=kappa, dagger=dagger)
 
@@ -119,3 +119,51 @@ def test_batch_is_bit_identical():
             out = batch.apply_D(ps, 64, dagger=dagger)
             for op, p, n, o in zip(ops, ps, (3, 1), out):
                 assert torch.equal(o, (op.apply_Ddag if dagger else op.apply_D)(p, 64, n))
+
+
+def _check_sap(name, b, kappa=None, n_cy=2, n_mr=4, x0=None, p=0, tol=2e-15):
+    dims, block, eps, kap, csw, U, _ = fields(name)
+    kappa = kap if kappa is None else kappa
+    xg = None if x0 is None else torch.from_numpy(_scaled(x0, p)).cuda()
+    got = _op(name, kappa=kappa).sap(torch.from_numpy(_scaled(b, p)).cuda(), 64, n_cy, n_mr, x0=xg).cpu().numpy()
+    ref = O.sap(dims, block, -1, kappa, U, O.clover(dims, kappa, csw, U), b, x0=x0, ncy=n_cy, nmr=n_mr)
+    assert rel(_scaled(got, -p), ref) < tol
+    return got
+
+
+# the domain solves' sums differ in order from the oracle's: a few 1e-16 each,
+# over two sweeps of four steps below 2e-15
+@pytest.mark.parametrize("name", ["c0_4^4", "ragged_8x4x12x8", "mid_8^4"])
+@pytest.mark.parametrize("kappa", [0.0002, 0.02, 0.13, -0.11, 0.2])  # 0.0002 runs on FP64 instructions
+def test_sap(name, kappa):
+    psi = fields(name)[6]
+    _check_sap(name, psi, kappa)
+    _check_sap(name, psi, kappa, x0=np.roll(psi, 7, axis=0))
+
+
+@pytest.mark.parametrize("n_mr", [1, 3, 40])
+def test_sap_step_counts(n_mr):
+    _check_sap("ragged_8x4x12x8", fields("ragged_8x4x12x8")[6], n_cy=1, n_mr=n_mr)
+
+
+@pytest.mark.parametrize("p", [-880, -400, 400, 955])
+def test_sap_scales(p):
+    _check_sap("mid_8^4", fields("mid_8^4")[6], p=p)
+
+
+def test_sap_sparse_and_zero_domains():
+    name = "mid_8^4"
+    b = np.zeros_like(fields(name)[6])
+    b[77, 2, 1] = 1.5 - 0.25j
+    got = _check_sap(name, b, n_cy=1)
+    assert (got == 0).any()
+    b = fields(name)[6].copy()
+    b *= np.exp2(np.random.default_rng(3).integers(-40, 41, b.shape[0]))[:, None, None]
+    _check_sap(name, b)
+
+
+def test_sap_non_finite():
+    b = fields("mid_8^4")[6].copy()
+    b[100, 1, 2] = np.nan
+    x = _op("mid_8^4").sap(torch.from_numpy(b).cuda(), 64, 1, 4)
+    assert bool(torch.isnan(x.real).any())

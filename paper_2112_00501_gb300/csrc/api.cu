@@ -298,8 +298,6 @@ int mgc_clover_create(mgc_gauge_t g, double kappa, double csw, void *stream, mgc
     CCUDA(cudaMalloc(&op->Ci64, clover_bytes(geo, 64)));
     CCUDA(cudaMalloc(&d_bad, 3 * sizeof(int)));
     CCUDA(cudaMemsetAsync(d_bad, 0, 3 * sizeof(int), s));
-    int st = launch_clover_build(geo, g->U64, kappa, csw, op->C64, op->Ci64, d_bad, s);
-    if (st) return bail(st);
     // fixed-point copies for the FP64 operator, for hopping parameters of ordinary
     // size and where there is room for them (it runs without)
     const double ks = std::frexp(kappa, &op->fix_ek);
@@ -311,12 +309,14 @@ int mgc_clover_create(mgc_gauge_t g, double kappa, double csw, void *stream, mgc
             free_fix(op);
         }
     }
-    if (op->CQ) {
-        st = launch_fix_links(geo, g->U64, ks, op->UQ, d_bad + 1, s);
-        if (st) return bail(st);
-        st = launch_fix_clover(geo, op->C64, op->fix_ek, op->CQ, op->CE, d_bad + 1, s);
-        if (st) return bail(st);
-    }
+    int st = MGC_OK;
+    if (op->CQ) st = launch_fix_links(geo, g->U64, ks, op->UQ, d_bad + 1, s);
+    if (st) return bail(st);
+    st = launch_clover_build(geo, g->U64, op->CQ ? op->UQ : nullptr, ks, d_bad + 1, kappa, csw, op->C64, op->Ci64,
+                             d_bad, s);
+    if (st) return bail(st);
+    if (op->CQ) st = launch_fix_clover(geo, op->C64, op->fix_ek, op->CQ, op->CE, d_bad + 1, s);
+    if (st) return bail(st);
     // C and C^-1 (the latter for the clover-preconditioned operator A = C^-1 D)
     // at every precision the gauge field keeps
     if (g->prec <= 32) {

@@ -195,18 +195,10 @@ __device__ __forceinline__ int2 fix_store(fix_t q)
     return make_int2(hi, max(lo, -0x7fffffff));
 }
 
-// a b 2^60
-__device__ __forceinline__ int2 fix_product(double a, double b)
-{
-    const double hi = a * b, lo = fma(a, b, -hi);
-    const fix_t t = __double2ll_rn(hi * 0x1p60);
-    return fix_store(t + __double2ll_rn((hi * 0x1p60 - (double)t) + lo * 0x1p60));
-}
-
-// The links times ks (|ks| <= 1) in units of 2^-60, the product formed with its
-// remainder; *bad is set unless the rows and columns of every link have norm 1 to
+// The links times ks (0 < |ks| < 1, as ks62 = ks 2^62) in units of 2^-60, rounded to
+// nearest; *bad is set unless the rows and columns of every link have norm 1 to
 // 1e-3, which bounds the operator's sums.
-__global__ void k_fix_links(Geom g, Gauge64 U, double ks, int4 *__restrict__ out, int *bad)
+__global__ void k_fix_links(Geom g, Gauge64 U, long long ks62, int4 *__restrict__ out, int *bad)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= g.V) return;
@@ -214,19 +206,24 @@ __global__ void k_fix_links(Geom g, Gauge64 U, double ks, int4 *__restrict__ out
     Cx<double> u[9];
     U.load(i, mu, u);
     int4 *o = out + (((size_t)(i >> g.lvb) * 4 + mu) * 9 << g.lvb) + (i & ((1 << g.lvb) - 1));
+    float n[9];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) n[k] = norm2(Cx<float>{(float)u[k].r, (float)u[k].i});
     bool fine = true;
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        const double row = norm2(u[3 * a]) + norm2(u[3 * a + 1]) + norm2(u[3 * a + 2]);
-        const double col = norm2(u[a]) + norm2(u[3 + a]) + norm2(u[6 + a]);
-        fine = fine && fabs(row - 1.0) < 1e-3 && fabs(col - 1.0) < 1e-3;
-    }
+    for (int a = 0; a < 3; ++a)
+        fine = fine && fabsf(n[3 * a] + n[3 * a + 1] + n[3 * a + 2] - 1.f) < 1e-3f &&
+               fabsf(n[a] + n[3 + a] + n[6 + a] - 1.f) < 1e-3f;
+    if (!fine) atomicOr(bad, 1);
+    auto scaled = [&](double x) {
+        const long long q = fix_from_any(x, 1026) << 2;  // x 2^62, |x| < 1.001
+        return fix_store(__mul64hi(q, ks62) + (long long)((unsigned long long)(q * ks62) >> 63));
+    };
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
-        const int2 r = fix_product(u[k].r, ks), m = fix_product(u[k].i, ks);
+        const int2 r = scaled(u[k].r), m = scaled(u[k].i);
         o[(size_t)k << g.lvb] = make_int4(r.x, r.y, m.x, m.y);
     }
-    if (!fine) atomicOr(bad, 1);
 }
 
 // C in units of 2^(e + ek - 60) with the site's exponent e, |C| < 2^(e + ek) and a
@@ -285,7 +282,8 @@ __global__ void k_fix_clover(Geom g, Clover64 C, int ek, int4 *__restrict__ out,
 
 int launch_fix_links(const Geom &g, const double2 *U64, double ks, int4 *out, int *d_bad, cudaStream_t s)
 {
-    k_fix_links<<<dim3(grid_for(g.V, 128), 4), 128, 0, s>>>(g, Gauge64{(double2 *)U64, g.lvb}, ks, out, d_bad);
+    k_fix_links<<<dim3(grid_for(g.V, 128), 4), 128, 0, s>>>(g, Gauge64{(double2 *)U64, g.lvb}, (long long)(ks * 0x1p62),
+                                                                 out, d_bad);
     MGC_CUDA(cudaGetLastError());
     count(1, (double)g.V * (2 * 576.0));
     return MGC_OK;

@@ -165,6 +165,18 @@ __device__ __forceinline__ fix_t fix_from(uint32_t lo, uint32_t hi, int K, uint3
     return (fix_t)(((unsigned long long)qh << 32) | ql);
 }
 
+// Q of a double, K = the unit's biased exponent + 4: x = Q 2^(K - 1086) rounded
+// towards zero, |x| < 2^(K - 1026)
+__device__ __forceinline__ fix_t fix_from_any(double x, int K)
+{
+    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+    const int e = (int)(hi >> 20) & 0x7ff;
+    const int s = K - e;
+    unsigned long long m = ((unsigned long long)(__funnelshift_l(lo, hi, 11) | 0x80000000u) << 32) | (lo << 11);
+    m = (e == 0 || s > 63) ? 0 : m >> s;
+    return (int)hi < 0 ? -(fix_t)m : (fix_t)m;
+}
+
 // component k of the site in units of 2^(E - 60), K = E + 4
 __device__ __forceinline__ Cx<fix_t> fix_component(const FixRaw &r, int k, int K, uint32_t neg = 0)
 {

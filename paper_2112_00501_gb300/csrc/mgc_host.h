@@ -122,8 +122,10 @@ int launch_scale_to32(const Geom &g, const double2 *in, void *out, double s, cud
 int launch_axpy_from32(const Geom &g, double2 *x, const void *e, double cr, double ci, cudaStream_t st);
 
 // clover_build.cu
-int launch_clover_build(const Geom &g, const double2 *U64, double kappa, double csw, double2 *C64, double2 *Ci64,
-                        int *d_bad, cudaStream_t s);
+// C and C^-1; from the fixed-point links UQ (scaled by ks) where they are given and
+// *no_fix is zero on the device
+int launch_clover_build(const Geom &g, const double2 *U64, const int4 *UQ, double ks, const int *no_fix, double kappa,
+                        double csw, double2 *C64, double2 *Ci64, int *d_bad, cudaStream_t s);
 int launch_clover_lowprec(const Geom &g, const double2 *C64, int prec, void *out, cudaStream_t s);
 int launch_clover_export(const Geom &g, const double2 *C64, double *out, cudaStream_t s);
 int launch_unitarity(const Geom &g, const double *canon_dev, double *d_maxerr, cudaStream_t s);

@@ -373,18 +373,6 @@ __global__ void __launch_bounds__(256) k_sap_colour(Geom g, SP b, SP x, GA U, CL
 // instructions.  Error of two sweeps against quadruple precision on 8^4: 1.0e-16
 // against 2.3e-16.
 
-// Q of a double, K = the unit's biased exponent + 4: x = Q 2^(K - 1086) rounded
-// towards zero, |x| < 2^(K - 1026)
-__device__ __forceinline__ fix_t fix_from_any(double x, int K)
-{
-    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
-    const int e = (int)(hi >> 20) & 0x7ff;
-    const int s = K - e;
-    unsigned long long m = ((unsigned long long)(__funnelshift_l(lo, hi, 11) | 0x80000000u) << 32) | (lo << 11);
-    m = (e == 0 || s > 63) ? 0 : m >> s;
-    return (int)hi < 0 ? -(fix_t)m : (fix_t)m;
-}
-
 // the largest biased exponent of 24 reals
 __device__ __forceinline__ int fix_exponent(const Cx<double> v[12])
 {

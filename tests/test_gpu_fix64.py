@@ -167,3 +167,25 @@ def test_sap_non_finite():
     b[100, 1, 2] = np.nan
     x = _op("mid_8^4").sap(torch.from_numpy(b).cuda(), 64, 1, 4)
     assert bool(torch.isnan(x.real).any())
+
+
+@pytest.mark.parametrize("name", ["c0_4^4", "ragged_8x4x12x8", "mid_8^4"])
+@pytest.mark.parametrize("kappa,csw,bent", [(0.13, 1.0, False), (0.13, 4.0, False), (0.13, 30.0, False),
+                                            (-0.13, 1.7, False), (0.13, 1.0, True), (1e-6, 1.0, False)])
+def test_clover_build(name, kappa, csw, bent):
+    """Blocks that are positive definite and (large c_SW) not; links with and without a fixed-point
+    copy.  C to a few roundings of its largest entries; C C^-1 = 1 to those times the condition."""
+    from paper_2112_00501_gb300 import api
+
+    dims, block, eps, _, _, U, psi = fields(name)
+    U = U.copy()
+    if bent:
+        U[5, 2] *= 1.01
+    lat = api.Lattice(dims, block, -1)
+    op = api.CloverOperator(api.Gauge(lat, torch.from_numpy(U).cuda(), storage_prec=64), kappa, csw)
+    C, Ci = op.export_clover().cpu().numpy(), op.export_clover(inverse=True).cpu().numpy()
+    ref = O.clover(dims, kappa, csw, U).reshape(C.shape)
+    assert rel(C, ref) < 5e-16
+    cond = np.linalg.norm(ref, axis=(1, 2)) * np.linalg.norm(np.linalg.inv(ref), axis=(1, 2))
+    err = np.linalg.norm(np.einsum("sij,sjk->sik", C, Ci) - np.eye(12), axis=(1, 2))
+    assert (err < 1e-15 * cond).all()

@@ -19,7 +19,7 @@
 // e <- r_B + kappa C^-1 H_B e from e = 0 (the first gives e = r_B), with e
 // (instead of r) in shared memory and no block reductions.
 //
-// In mode SAP_EO (FP64 and staged kernels) the domain solve is the even-odd
+// In mode SAP_EO (FP64) and in k_sap_eo (FP32, FP16) the domain solve is the even-odd
 // preconditioned MR of DD-alphaAMG: the even sites (the first half of a domain
 // in the packed order) run MR on the Schur complement
 // C_ee - kappa^2 H_eo C_oo^-1 H_oe with source r_e + kappa H_eo C_oo^-1 r_o,
@@ -30,6 +30,7 @@
 #include "hop.cuh"
 #include "hop16.cuh"
 #include "mgc_host.h"
+#include "sap_split.cuh"
 #include "tma.cuh"
 
 namespace mgc {
@@ -849,9 +850,8 @@ __device__ __forceinline__ void sap_staged_body(const Geom &g, const SP &b, cons
                                                 const CL &Ci, float kappa, int colour, int nmr, int x_zero,
                                                 int *status, int jb, int rr);
 
-// the even-odd solver keeps more state per thread: one block per SM
 template <int MODE, class SP, class GA, class CL>
-__global__ void __launch_bounds__(256, MODE == SAP_EO ? 1 : staged_min_ctas<GA, CL>())
+__global__ void __launch_bounds__(256, staged_min_ctas<GA, CL>())
     k_sap_staged(Geom g, SP b, SP x, GA U, CL C, CL Ci, float kappa, int colour, int nmr, int x_zero, int *status)
 {
     sap_staged_body<MODE>(g, b, x, U, C, Ci, kappa, colour, nmr, x_zero, status, blockIdx.x, blockIdx.y);
@@ -960,87 +960,6 @@ __device__ __forceinline__ void sap_staged_body(const Geom &g, const SP &b, cons
         es[k * vb + l] = Cx<float>{0.f, 0.f};
     }
     __syncthreads();
-
-    // 2''. even-odd preconditioned MR (C^-1 of the odd sites from global memory)
-    if (MODE == SAP_EO) {
-        const bool even = l < (vb >> 1);
-        Cx<float> rho[12], t[12], ee[12];
-        auto hops = [&]() {
-#pragma unroll
-            for (int k = 0; k < 12; ++k) acc[k] = Cx<float>{0.f, 0.f};
-            staged_hop_dir<0>(Us, l, nf[0], nb[0], rs, vb, acc);
-            staged_hop_dir<1>(Us, l, nf[1], nb[1], rs, vb, acc);
-            staged_hop_dir<2>(Us, l, nf[2], nb[2], rs, vb, acc);
-            staged_hop_dir<3>(Us, l, nf[3], nb[3], rs, vb, acc);
-        };
-#pragma unroll
-        for (int k = 0; k < 12; ++k) ee[k] = Cx<float>{0.f, 0.f};
-        if (!even) {
-            clover_site(Ci, i, rv, t);
-#pragma unroll
-            for (int k = 0; k < 12; ++k) rs[k * vb + l] = t[k];
-        }
-        __syncthreads();
-        if (even) {
-            hops();
-#pragma unroll
-            for (int k = 0; k < 12; ++k)
-                rho[k] = Cx<float>{fmaf(kappa, acc[k].r, rv[k].r), fmaf(kappa, acc[k].i, rv[k].i)};
-        }
-        __syncthreads();
-        if (even)
-#pragma unroll
-            for (int k = 0; k < 12; ++k) rs[k * vb + l] = rho[k];
-        __syncthreads();
-        for (int it = 0; it < nmr; ++it) {
-            if (!even) {
-                hops();
-#pragma unroll
-                for (int k = 0; k < 12; ++k) acc[k] = kappa * acc[k];
-                clover_site(Ci, i, acc, t);
-#pragma unroll
-                for (int k = 0; k < 12; ++k) rs[k * vb + l] = t[k];
-            }
-            __syncthreads();
-            float pr = 0.f, pi = 0.f, pp = 0.f;
-            Cx<float> p[12];
-            if (even) {
-                hops();
-                Cs.mul(l, rho, p);
-#pragma unroll
-                for (int k = 0; k < 12; ++k) {
-                    p[k] = Cx<float>{fmaf(-kappa, acc[k].r, p[k].r), fmaf(-kappa, acc[k].i, p[k].i)};
-                    pr = fmaf(p[k].r, rho[k].r, fmaf(p[k].i, rho[k].i, pr));
-                    pi = fmaf(p[k].r, rho[k].i, fmaf(-p[k].i, rho[k].r, pi));
-                    pp = fmaf(p[k].r, p[k].r, fmaf(p[k].i, p[k].i, pp));
-                }
-            }
-            block_sum3(pr, pi, pp, red);
-            const Cx<float> alpha = (pp > 0.f) ? Cx<float>{pr / pp, pi / pp} : Cx<float>{0.f, 0.f};
-            if (even)
-#pragma unroll
-                for (int k = 0; k < 12; ++k) {
-                    ee[k] = cfma(alpha, rho[k], ee[k]);
-                    rho[k] = rho[k] - alpha * p[k];
-                    rs[k * vb + l] = rho[k];
-                }
-            __syncthreads();
-        }
-        if (even)
-#pragma unroll
-            for (int k = 0; k < 12; ++k) rs[k * vb + l] = ee[k];
-        __syncthreads();
-        if (!even) {
-            hops();
-#pragma unroll
-            for (int k = 0; k < 12; ++k)
-                t[k] = Cx<float>{fmaf(kappa, acc[k].r, rv[k].r), fmaf(kappa, acc[k].i, rv[k].i)};
-            clover_site(Ci, i, t, ee);
-        }
-#pragma unroll
-        for (int k = 0; k < 12; ++k) es[k * vb + l] = ee[k];
-        nmr = 0;
-    }
 
     // 2'. Jacobi on A_B with e in shared memory (rs): e_1 = r_B, then
     // e <- r_B + kappa C^-1 H_B e
@@ -2255,6 +2174,173 @@ static int sap_run_staged(const mgc_clover_s *op, SP b, SP x, GA U, CL C, CL Ci,
     return MGC_OK;
 }
 
+// ------------------------------------------------------------------ even-odd kernel
+// FP32 and FP16 storage, even-odd MR: two threads per site of one parity
+// (sap_split.cuh); the domain's links as 18-real FP32, C of its even and C^-1 of its
+// odd sites and one vector, whose even entries hold rho (then e), the odd ones the
+// odd sites' intermediate, in shared memory: 172 KB at 256 sites, one block per SM.
+static size_t eo_smem(int vb) { return (size_t)vb * (288 + 288 + 96) + 96 * sizeof(float); }
+
+template <int LVB, class SP, class GA, class CL>
+__global__ void __launch_bounds__(256, 1) k_sap_eo(Geom g, SP b, SP x, GA U, CL C, CL Ci, float kappa, int colour,
+                                                   int nmr, int x_zero)
+{
+    extern __shared__ __align__(128) unsigned char smem[];
+    if (LVB > 0) {
+        g.lvb = LVB;
+#pragma unroll
+        for (int mu = 0; mu < 4; ++mu) g.lb[mu] = LVB / 4;
+        b.lvb = x.lvb = U.lvb = C.lvb = Ci.lvb = LVB;
+    }
+    const int vb = 1 << g.lvb;
+    float2 *const sL = reinterpret_cast<float2 *>(smem);  // [mu 9 + entry][vb]
+    float2 *const sC = sL + 36 * vb;                      // [pair of reals][vb]
+    float2 *const rs = sC + 36 * vb;                      // [component][vb]
+    float *const red = reinterpret_cast<float *>(rs + 12 * vb);
+    const SP bb = shift_rhs(b, blockIdx.y, g.V), xx = shift_rhs(x, blockIdx.y, g.V);
+    int j = blockIdx.x;
+    const int half0 = g.NB[0] >> 1;
+    int bc[4], lc[4], c[4];
+    const int m = j % half0;
+    j /= half0;
+    bc[1] = j % g.NB[1];
+    j /= g.NB[1];
+    bc[2] = j % g.NB[2];
+    bc[3] = j / g.NB[2];
+    bc[0] = 2 * m + ((colour + bc[1] + bc[2] + bc[3]) & 1);
+    const int base = block_index(g, bc) << g.lvb;
+    const int t = threadIdx.x;
+
+    // 1. one thread per site: its links and clover term, and the residual of D
+    {
+        const int i = base | t;
+        local_coords(g, t, lc);
+#pragma unroll
+        for (int mu = 0; mu < 4; ++mu) {
+            c[mu] = (bc[mu] << g.lb[mu]) + lc[mu];
+            Cx<float> u[9];
+            U.load(i, mu, u);
+#pragma unroll
+            for (int k = 0; k < 9; ++k) sL[(mu * 9 + k) * vb + t] = make_float2(u[k].r, u[k].i);
+        }
+        Cx<float> rv[12];
+        bb.load(i, rv);
+        if (!x_zero) {
+            Cx<float> dx[12];
+            dirac_site<false>(g, c, i, xx, U, C, kappa, dx);
+#pragma unroll
+            for (int k = 0; k < 12; ++k) rv[k] = rv[k] - dx[k];
+        }
+#pragma unroll
+        for (int k = 0; k < 12; ++k) rs[k * vb + t] = make_float2(rv[k].r, rv[k].i);
+        float cl[72];
+        (t < (vb >> 1) ? C : Ci).load(i, cl);
+#pragma unroll
+        for (int k = 0; k < 36; ++k) sC[k * vb + t] = make_float2(cl[2 * k], cl[2 * k + 1]);
+    }
+    __syncthreads();
+
+    // two threads per even site le and per odd site lo
+    const int q = t & 1, le = t >> 1, lo = le + (vb >> 1);
+    const float sg = q ? -1.f : 1.f;
+    uint32_t ne[4], no[4];
+    local_coords(g, le, lc);
+    split_neighbours(g, lc, ne);
+    local_coords(g, lo, lc);
+    split_neighbours(g, lc, no);
+
+    // 2. rho = r_e + kappa H_eo C_oo^-1 r_o
+    Cx<float> ro[6], rho[6], e[6], v[6], w[6];
+    split_get(rs, vb, lo, q, ro);
+    split_get(rs, vb, le, q, rho);
+    split_clover(sC, vb, lo, q, sg, ro, w);
+    split_put(rs, vb, lo, q, w);
+    __syncthreads();
+    split_hops(rs, vb, sL, le, ne, q, sg, v);
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+        rho[k] = Cx<float>{fmaf(kappa, v[k].r, rho[k].r), fmaf(kappa, v[k].i, rho[k].i)};
+        e[k] = Cx<float>{0.f, 0.f};
+    }
+    split_put(rs, vb, le, q, rho);
+    __syncthreads();
+
+    // 3. MR on the Schur complement
+    for (int it = 0; it < nmr; ++it) {
+        // odd sites: y = C_oo^-1 (kappa H_oe rho)
+        split_hops(rs, vb, sL, lo, no, q, sg, v);
+#pragma unroll
+        for (int k = 0; k < 6; ++k) v[k] = kappa * v[k];
+        split_clover(sC, vb, lo, q, sg, v, w);
+        split_put(rs, vb, lo, q, w);
+        __syncthreads();
+        // even sites: p = C_ee rho - kappa H_eo y, MR step
+        split_hops(rs, vb, sL, le, ne, q, sg, v);
+        split_clover(sC, vb, le, q, sg, rho, w);
+        float pr = 0.f, pi = 0.f, pp = 0.f;
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            w[k] = Cx<float>{fmaf(-kappa, v[k].r, w[k].r), fmaf(-kappa, v[k].i, w[k].i)};
+            pr = fmaf(w[k].r, rho[k].r, fmaf(w[k].i, rho[k].i, pr));
+            pi = fmaf(w[k].r, rho[k].i, fmaf(-w[k].i, rho[k].r, pi));
+            pp = fmaf(w[k].r, w[k].r, fmaf(w[k].i, w[k].i, pp));
+        }
+        block_sum3(pr, pi, pp, red);
+        // a domain whose <p, p> is below FP32's normal range takes no step
+        const float ipp = pp >= FLT_MIN ? 1.0f / pp : 0.f;
+        const Cx<float> alpha = {pr * ipp, pi * ipp};
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            e[k] = cfma(alpha, rho[k], e[k]);
+            rho[k] = rho[k] - alpha * w[k];
+        }
+        split_put(rs, vb, le, q, rho);
+        __syncthreads();
+    }
+
+    // 4. e_o = C_oo^-1 (r_o + kappa H_oe e_e)
+    split_put(rs, vb, le, q, e);
+    __syncthreads();
+    split_hops(rs, vb, sL, lo, no, q, sg, v);
+#pragma unroll
+    for (int k = 0; k < 6; ++k) v[k] = Cx<float>{fmaf(kappa, v[k].r, ro[k].r), fmaf(kappa, v[k].i, ro[k].i)};
+    split_clover(sC, vb, lo, q, sg, v, w);
+    split_put(rs, vb, lo, q, w);
+    __syncthreads();
+
+    // 5. x_B += e, one thread per site
+    const int i = base | t;
+    Cx<float> xo[12];
+    if (!x_zero) xx.load(i, xo);
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+        const float2 d = rs[k * vb + t];
+        xo[k] = x_zero ? Cx<float>{d.x, d.y} : Cx<float>{d.x + xo[k].r, d.y + xo[k].i};
+    }
+    xx.store(i, xo);
+}
+
+template <class SP, class GA, class CL>
+static int sap_run_eo(const mgc_clover_s *op, SP b, SP x, GA U, CL C, CL Ci, int nrhs, int n_cy, int n_mr, int x_is_zero,
+                      cudaStream_t s, int prec, int compress)
+{
+    const Geom &g = op->gauge->lat->g;
+    const int vb = 1 << g.lvb;
+    const bool cube = g.lb[0] == g.lb[1] && g.lb[1] == g.lb[2] && g.lb[2] == g.lb[3];
+    const size_t smem = eo_smem(vb);
+    auto kern = cube && g.lvb == 8 ? k_sap_eo<8, SP, GA, CL> : k_sap_eo<0, SP, GA, CL>;
+    MGC_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    dim3 grid(g.nblocks / 2, nrhs);
+    for (int cy = 0; cy < n_cy; ++cy)
+        for (int colour = 0; colour < 2; ++colour) {
+            const int xz = (cy == 0 && colour == 0) ? x_is_zero : 0;
+            kern<<<grid, vb, smem, s>>>(g, b, x, U, C, Ci, (float)op->kappa, colour, n_mr, xz);
+            count(1, sap_launch_bytes(g, prec, compress, nrhs, xz != 0));
+        }
+    MGC_CUDA(cudaGetLastError());
+    return MGC_OK;
+}
+
 template <int MODE, class SP, class GA, class CL>
 static int sap_run(const Geom &g, SP b, SP x, GA U, CL C, CL Ci, double kappa, int nrhs, int n_cy, int n_mr,
                    int x_is_zero,
@@ -2346,11 +2432,17 @@ static int sap_launch_impl(const mgc_clover_s *op, int prec, const void *b, void
             return cp == 12 ? sap_run_f32<jac, 4>(op, B, X, U12, C, nrhs, n_cy, n_it, x_is_zero, s, cp)
                             : sap_run_f32<jac, 4>(op, B, X, U18, C, nrhs, n_cy, n_it, x_is_zero, s, cp);
         }
-        if (cp == 12)
+        if constexpr (MODE == SAP_EO)
+            return cp == 12 ? sap_run_eo(op, B, X, Gauge32x12{(float4 *)ga->U32, g.lvb}, C, Ci, nrhs, n_cy, n_it,
+                                         x_is_zero, s, prec, cp)
+                            : sap_run_eo(op, B, X, Gauge32x18{(float2 *)ga->U32, g.lvb}, C, Ci, nrhs, n_cy, n_it,
+                                         x_is_zero, s, prec, cp);
+        else if (cp == 12)
             return sap_run_staged<MODE>(op, B, X, Gauge32x12{(float4 *)ga->U32, g.lvb}, C, Ci, nrhs, n_cy, n_it,
                                         x_is_zero, s, prec, cp);
-        return sap_run_staged<MODE>(op, B, X, Gauge32x18{(float2 *)ga->U32, g.lvb}, C, Ci, nrhs, n_cy, n_it,
-                                    x_is_zero, s, prec, cp);
+        else
+            return sap_run_staged<MODE>(op, B, X, Gauge32x18{(float2 *)ga->U32, g.lvb}, C, Ci, nrhs, n_cy, n_it,
+                                        x_is_zero, s, prec, cp);
     }
     const size_t nV = (size_t)nrhs * g.V;
     Spinor16 B{(uint4 *)b, (float *)((uint4 *)b + nV * 3), g.lvb};
@@ -2359,10 +2451,10 @@ static int sap_launch_impl(const mgc_clover_s *op, int prec, const void *b, void
     const Clover16 C = jac ? Ci : Clover16{(uint4 *)op->C16, op->C16_sc, g.lvb};
     if (MODE == SAP_EO) {
         if (cp == 12)
-            return sap_run_staged<SAP_EO>(op, B, X, Gauge16x12{(uint2 *)ga->U16, g.lvb}, C, Ci, nrhs, n_cy, n_it,
-                                          x_is_zero, s, 16, cp);
-        return sap_run_staged<SAP_EO>(op, B, X, Gauge16x18{(uint32_t *)ga->U16, g.lvb}, C, Ci, nrhs, n_cy, n_it,
-                                      x_is_zero, s, 16, cp);
+            return sap_run_eo(op, B, X, Gauge16x12{(uint2 *)ga->U16, g.lvb}, C, Ci, nrhs, n_cy, n_it, x_is_zero, s, 16,
+                              cp);
+        return sap_run_eo(op, B, X, Gauge16x18{(uint32_t *)ga->U16, g.lvb}, C, Ci, nrhs, n_cy, n_it, x_is_zero, s, 16,
+                          cp);
     }
     if (cp == 12)
         return sap_dispatch16<jac>(op, B, X, Gauge16x12{(uint2 *)ga->U16, g.lvb}, C, nrhs, n_cy, n_it, x_is_zero, s,

@@ -174,7 +174,9 @@ def test_sap_non_finite():
                                             (-0.13, 1.7, False), (0.13, 1.0, True), (1e-6, 1.0, False)])
 def test_clover_build(name, kappa, csw, bent):
     """Blocks that are positive definite and (large c_SW) not; links with and without a fixed-point
-    copy.  C to a few roundings of its largest entries; C C^-1 = 1 to those times the condition."""
+    copy.  C to a few roundings of its largest entries; C C^-1 = 1 to the residual bound of an
+    elimination on 6 x 6 complex blocks, 10 n u cond = 6.7e-15 cond (u = 1.1e-16); the blocks that
+    are not definite go through Gauss-Jordan elimination, whose residual carries the condition twice."""
     from paper_2112_00501_gb300 import api
 
     dims, block, eps, _, _, U, psi = fields(name)
@@ -188,4 +190,4 @@ def test_clover_build(name, kappa, csw, bent):
     assert rel(C, ref) < 5e-16
     cond = np.linalg.norm(ref, axis=(1, 2)) * np.linalg.norm(np.linalg.inv(ref), axis=(1, 2))
     err = np.linalg.norm(np.einsum("sij,sjk->sik", C, Ci) - np.eye(12), axis=(1, 2))
-    assert (err < 1e-15 * cond).all()
+    assert (err < 6.7e-15 * cond * (cond if csw > 4 else 1.0)).all()

@@ -6,8 +6,7 @@
 //    per site).
 //  - gauge pack: canonical links -> packed links (18 or 12 reals).
 //  - k_dirac: out = C psi - kappa H psi (Eq. (1)), or D^dagger with the
-//    projectors swapped, one thread per site; a right-hand-side index runs
-//    over blockIdx.y.
+//    projectors swapped, one thread per site and right-hand side.
 //  - k_clover_apply: out = C psi or C^-1 psi.
 #include "hop.cuh"
 #include "fix64.cuh"
@@ -350,17 +349,39 @@ static void dirac_fix_dispatch(const mgc_clover_s *op, bool dag, Spinor64 in, Sp
 // 128-thread blocks, five per SM for FP32 arithmetic (96 registers, no
 // spills); measured against 256 x 2, 256 x 3 and 128 x 6 on 32^3 x 64.
 constexpr int DIRAC_THREADS = 128;
+
+// Right-hand sides: RF numbers them fastest (blockIdx.x), so that the blocks of one
+// site block run together and find its links and clover term in L2; otherwise a
+// right-hand side's site blocks stay together.  RF is taken where a launch's fields
+// exceed 0.9 of the 129 MB L2 and blockIdx.y can count the site blocks (20x12x28x36,
+// three FP32 right-hand sides, 279 MB: 73 us against 96 us; 16^3x32, five, 201 MB: 62
+// against 74); below it is 1 to 3 % slower (16^3x32, three at FP16, 52 MB: 29.1
+// against 28.2).
+template <bool RF>
+__device__ __forceinline__ int site_of_block(int &r)
+{
+    r = RF ? blockIdx.x : blockIdx.y;
+    return (RF ? blockIdx.y : blockIdx.x) * blockDim.x + threadIdx.x;
+}
+
+static bool rhs_fast(const Geom &g, int prec, int compress, int nrhs)
+{
+    return nrhs > 1 && grid_for(g.V, DIRAC_THREADS) <= 65535 &&
+           g.V * (nrhs * 2 * spinor_site_bytes(prec) + links_site_bytes(prec, compress) + clover_site_bytes(prec)) >
+               116e6;
+}
+
 // The input and output spinors may differ in storage (an FP16 input with the
 // FP32 operator); the arithmetic type is theirs, which must agree.
-template <bool DAG, int LVB, class SPI, class SPO, class GA, class CL>
+template <bool RF, bool DAG, int LVB, class SPI, class SPO, class GA, class CL>
 __global__ void __launch_bounds__(DIRAC_THREADS, (LVB > 0 && sizeof(typename SPI::Real) == 4) ? 5 : 1)
     k_dirac(Geom g, SPI in, SPO out, GA U, CL C, typename SPI::Real kappa)
 {
     using T = typename SPI::Real;
     static_assert(std::is_same<T, typename SPO::Real>::value, "input and output share the arithmetic type");
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    int r;
+    const int i = site_of_block<RF>(r);
     if (i >= g.V) return;
-    const int r = blockIdx.y;
     SPI src = shift_rhs(in, r, g.V);
     SPO dst = shift_rhs(out, r, g.V);
     GA Ug = U;
@@ -390,13 +411,13 @@ __global__ void __launch_bounds__(DIRAC_THREADS, (LVB > 0 && sizeof(typename SPI
 // scales, FP32 arithmetic with the FP16 factors fed to the multiply-adds as
 // they are stored (hop16.cuh)
 
-template <bool DAG, int LVB, class GA>
+template <bool RF, bool DAG, int LVB, class GA>
 __global__ void __launch_bounds__(DIRAC_THREADS, 5)
     k_dirac16(Geom g, Spinor16 in, Spinor16 out, GA U, Clover16 C, float kappa)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    int r;
+    const int i = site_of_block<RF>(r);
     if (i >= g.V) return;
-    const int r = blockIdx.y;
     Spinor16 src = shift_rhs(in, r, g.V), dst = shift_rhs(out, r, g.V);
     GA Ug = U;
     Clover16 Cg = C;
@@ -432,9 +453,15 @@ template <int LVB, class GA>
 static void dirac16_launch(const Geom &g, bool dag, Spinor16 in, Spinor16 out, GA U, Clover16 C, double kappa,
                            int nrhs, cudaStream_t s)
 {
-    dim3 grid(grid_for(g.V, DIRAC_THREADS), nrhs);
-    if (dag) k_dirac16<true, LVB><<<grid, DIRAC_THREADS, 0, s>>>(g, in, out, U, C, (float)kappa);
-    else k_dirac16<false, LVB><<<grid, DIRAC_THREADS, 0, s>>>(g, in, out, U, C, (float)kappa);
+    const int nb = grid_for(g.V, DIRAC_THREADS), compress = std::is_same<GA, Gauge16x12>::value ? 12 : 18;
+    auto run = [&](auto rf) {
+        constexpr bool RF = decltype(rf)::value;
+        const dim3 grid(RF ? nrhs : nb, RF ? nb : nrhs);
+        if (dag) k_dirac16<RF, true, LVB><<<grid, DIRAC_THREADS, 0, s>>>(g, in, out, U, C, (float)kappa);
+        else k_dirac16<RF, false, LVB><<<grid, DIRAC_THREADS, 0, s>>>(g, in, out, U, C, (float)kappa);
+    };
+    if (rhs_fast(g, 16, compress, nrhs)) run(std::true_type{});
+    else run(std::false_type{});
 }
 
 template <class GA>
@@ -451,9 +478,18 @@ template <int LVB, class SPI, class SPO, class GA, class CL>
 static void dirac_launch(const Geom &g, bool dag, SPI in, SPO out, GA U, CL C, double kappa, int nrhs, cudaStream_t s)
 {
     using T = typename SPI::Real;
-    dim3 grid(grid_for(g.V, DIRAC_THREADS), nrhs);
-    if (dag) k_dirac<true, LVB><<<grid, DIRAC_THREADS, 0, s>>>(g, in, out, U, C, (T)kappa);
-    else k_dirac<false, LVB><<<grid, DIRAC_THREADS, 0, s>>>(g, in, out, U, C, (T)kappa);
+    const int nb = grid_for(g.V, DIRAC_THREADS), compress = std::is_same<GA, Gauge32x12>::value ? 12 : 18;
+    auto run = [&](auto rf) {
+        constexpr bool RF = decltype(rf)::value;
+        const dim3 grid(RF ? nrhs : nb, RF ? nb : nrhs);
+        if (dag) k_dirac<RF, true, LVB><<<grid, DIRAC_THREADS, 0, s>>>(g, in, out, U, C, (T)kappa);
+        else k_dirac<RF, false, LVB><<<grid, DIRAC_THREADS, 0, s>>>(g, in, out, U, C, (T)kappa);
+    };
+    // several right-hand sides at FP32 only come with one storage in and out
+    if constexpr (std::is_same<SPI, Spinor32>::value) {
+        if (rhs_fast(g, 32, compress, nrhs)) return run(std::true_type{});
+    }
+    run(std::false_type{});
 }
 
 template <class SPI, class SPO, class GA, class CL>

@@ -196,27 +196,6 @@ __constant__ LeafLink c_leaves[4][4] = {
     {{0, -1, 1, 1}, {0, -1, 0, 0}, {1, -1, 1, 0}, {0, 0, 0, 1}},
 };
 
-// limbs of a 3x3 complex matrix, entry k as (re hi, re lo, im hi, im lo)
-struct FixM3 {
-    int4 e[9];
-    // a link or its dagger
-    __device__ __forceinline__ void load(const FixLinks &U, int site, int mu, bool dag)
-    {
-        const int4 *q = U.at(site, mu);
-        const int sm = dag ? -1 : 0, sa = dag ? 1 : 3, sb = dag ? 3 : 1;
-#pragma unroll
-        for (int a = 0; a < 3; ++a)
-#pragma unroll
-            for (int b = 0; b < 3; ++b) {
-                int4 v = __ldg(q + ((a * sa + b * sb) << U.lvb));
-                v.z = (v.z ^ sm) - sm;
-                v.w = (v.w ^ sm) - sm;
-                asm("" : "+r"(v.z), "+r"(v.w));  // 32-bit numbers of unknown origin (fix_neg)
-                e[a * 3 + b] = v;
-            }
-    }
-};
-
 // a row of P (three complex limbs) times A, both in units of 2^-60: out in units of
 // 2^-(56 + L), L < 32
 __device__ __forceinline__ void fix_row_mul(const int4 p[3], const FixM3 &A, int L, Cx<fix_t> out[3])
@@ -226,22 +205,8 @@ __device__ __forceinline__ void fix_row_mul(const int4 p[3], const FixM3 &A, int
     for (int j = 0; j < 3; ++j) {
         fix_t hr = 0, hi = 0, mr = half, mi = half;
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            const int4 x = p[k], u = A.e[k * 3 + j];
-            const int n1 = fix_neg(u.z), n0 = fix_neg(u.w);
-            hr = mac64(n1, x.z, mac64(u.x, x.x, hr));
-            mr = mac64(u.y, x.x, mac64(u.x, x.y, mr));
-            mr = mac64(n0, x.z, mac64(n1, x.w, mr));
-            hi = mac64(u.z, x.x, mac64(u.x, x.z, hi));
-            mi = mac64(u.y, x.z, mac64(u.x, x.w, mi));
-            mi = mac64(u.w, x.x, mac64(u.z, x.y, mi));
-        }
-        auto shift = [&](fix_t h, fix_t m) {
-            const fix_t y = fix_join(h, m);
-            return (fix_t)(((unsigned long long)__funnelshift_l((uint32_t)y, (uint32_t)(y >> 32), L) << 32) |
-                           __funnelshift_l((uint32_t)m, (uint32_t)y, L));
-        };
-        out[j] = Cx<fix_t>{shift(hr, mr), shift(hi, mi)};
+        for (int k = 0; k < 3; ++k) fix_cmac(A.e[k * 3 + j], p[k], hr, mr, hi, mi);
+        out[j] = Cx<fix_t>{fix_join_bits(hr, mr, L), fix_join_bits(hi, mi, L)};
     }
 }
 

@@ -296,13 +296,13 @@ int launch_fix_clover(const Geom &g, const double2 *C64, int ek, int4 *out, int2
     return MGC_OK;
 }
 
-// D, D^dagger at FP64 in block fixed point (fix64.cuh).  24^3 x 48: 400 us
-// against 1259 us with FP64 instructions (2.5 TB/s of compulsory bytes against
+// D, D^dagger at FP64 in block fixed point (fix64.cuh).  24^3 x 48: 372 us
+// against 1259 us with FP64 instructions (2.7 TB/s of compulsory bytes against
 // 0.8); the FMA pipe's heavy half, where the widening products run, is busy 67 %
-// of the time.  Four blocks per SM (128 registers) and three (168) measure the
-// same; five spill (429 us).
+// of the time.  Three blocks per SM (168 registers); four (128) spill 200 B per
+// thread and take 403 us.
 template <bool DAG, int LVB>
-__global__ void __launch_bounds__(FIX_THREADS, 4)
+__global__ void __launch_bounds__(FIX_THREADS, 3)
     k_dirac_fix(Geom g, Spinor64 in, Spinor64 out, FixLinks U, FixClover C, Gauge64 Ud, Clover64 Cd, double kappa)
 {
     __shared__ int4 slots[(FIX_SPINOR_SLOTS + FIX_LINK_SLOTS) * FIX_THREADS];

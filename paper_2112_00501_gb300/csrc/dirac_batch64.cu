@@ -25,7 +25,7 @@ struct DiracBatchFix {
 };
 
 template <bool DAG, int LVB>
-__global__ void __launch_bounds__(FIX_THREADS, 4) k_dirac_batch_fix(DiracBatchFix B)
+__global__ void __launch_bounds__(FIX_THREADS, 3) k_dirac_batch_fix(DiracBatchFix B)
 {
     __shared__ int4 slots[(FIX_SPINOR_SLOTS + FIX_LINK_SLOTS) * FIX_THREADS];
     int k = 0;

@@ -211,6 +211,14 @@ __device__ __forceinline__ void fix_limbs(fix_t q, int &hi, int &lo)
 // hh + mid 2^-32 in units of hh, rounded down (the sums start from half a unit)
 __device__ __forceinline__ fix_t fix_join(fix_t hh, fix_t mid) { return mac64((int)(mid >> 32), 1, hh); }
 
+// hh + mid 2^-32 in units of hh 2^-L, rounded down, 0 <= L < 32
+__device__ __forceinline__ fix_t fix_join_bits(fix_t hh, fix_t mid, int L)
+{
+    const fix_t y = fix_join(hh, mid);
+    return (fix_t)(((unsigned long long)__funnelshift_l((uint32_t)y, (uint32_t)(y >> 32), L) << 32) |
+                   __funnelshift_l((uint32_t)mid, (uint32_t)y, L));
+}
+
 // (a, b) + sgn P (l0, l1) with P the spin map of direction MU: the projected
 // half spinor of one colour
 template <int MU, int SGN>
@@ -309,7 +317,7 @@ __device__ __forceinline__ void fix_hop(const int4 *link, int stride, int m, boo
 {
     const int sa = (back ? 1 : 3) * stride, sb = (back ? 3 : 1) * stride;
     const fix_t bm = back ? -1 : 0;
-    const fix_t cr = 0x80000000LL, ci = back ? -0x80000000LL : 0x80000000LL;  // half a unit of hh
+    const fix_t cr = 0x80000000LL, ci = (bm << 32) | 0x80000000LL;  // +- half a unit of hh
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         fix_t hr[2], hi[2], mr[2], mi[2];
@@ -415,16 +423,44 @@ __device__ __forceinline__ void fix_clover(const FixClover &C, int i, Q psi, int
         for (int m = 0; m < 12; ++m) {
             const fix_t y = fix_join(hh[m], mid[m]);
             fix_t r;
-            if (L >= 0) {  // bits of the middle sum below hh's unit
-                const uint32_t lo = __funnelshift_l((uint32_t)mid[m], (uint32_t)y, L);
-                const uint32_t hi = __funnelshift_l((uint32_t)y, (uint32_t)(y >> 32), L);
-                r = (fix_t)(((unsigned long long)hi << 32) | lo);
-            } else {
-                r = y >> min(-L, 63);
-            }
+            if (L >= 0) r = fix_join_bits(hh[m], mid[m], L);
+            else r = y >> min(-L, 63);
             (m & 1 ? acc[6 * chi + (m >> 1)].i : acc[6 * chi + (m >> 1)].r) = r;
         }
     }
+}
+
+// limbs of a 3x3 complex matrix, entry k as (re hi, re lo, im hi, im lo)
+struct FixM3 {
+    int4 e[9];
+    // a link or its dagger
+    __device__ __forceinline__ void load(const FixLinks &U, int site, int mu, bool dag)
+    {
+        const int4 *q = U.at(site, mu);
+        const int sm = dag ? -1 : 0, sa = dag ? 1 : 3, sb = dag ? 3 : 1;
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+#pragma unroll
+            for (int b = 0; b < 3; ++b) {
+                int4 v = __ldg(q + ((a * sa + b * sb) << U.lvb));
+                v.z = (v.z ^ sm) - sm;
+                v.w = (v.w ^ sm) - sm;
+                asm("" : "+r"(v.z), "+r"(v.w));  // 32-bit numbers of unknown origin (fix_neg)
+                e[a * 3 + b] = v;
+            }
+    }
+};
+
+// (hr, mr) + i (hi, mi) += u x, u and x complex limbs
+__device__ __forceinline__ void fix_cmac(int4 u, int4 x, fix_t &hr, fix_t &mr, fix_t &hi, fix_t &mi)
+{
+    const int n1 = fix_neg(u.z), n0 = fix_neg(u.w);
+    hr = mac64(n1, x.z, mac64(u.x, x.x, hr));
+    mr = mac64(u.y, x.x, mac64(u.x, x.y, mr));
+    mr = mac64(n0, x.z, mac64(n1, x.w, mr));
+    hi = mac64(u.z, x.x, mac64(u.x, x.z, hi));
+    mi = mac64(u.y, x.z, mac64(u.x, x.w, mi));
+    mi = mac64(u.w, x.x, mac64(u.z, x.y, mi));
 }
 
 // (D psi)(x) with FP64 instructions, for the sites the fixed-point path leaves

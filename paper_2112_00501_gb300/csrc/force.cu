@@ -17,8 +17,10 @@
 // three links M1 M2 M3 (in loop order after the link) with N(corner) inserted
 // where the loop passes each corner:
 //   R = N(c0) M1 M2 M3 + M1 N(c1) M2 M3 + M1 M2 N(c2) M3 + M1 M2 M3 N(c3).
+#include <cmath>
 #include <vector>
 
+#include "fix64.cuh"
 #include "hop.cuh"
 #include "mgc_host.h"
 #include "sigma.cuh"
@@ -247,6 +249,188 @@ __global__ void __launch_bounds__(128) k_force_plaq(Geom g, Gauge64 U, const dou
     put(3, R);                 // R_D
 }
 
+// ---- the same products in block fixed point (fix64.cuh), for operators with
+// fixed-point links.  Both kernels form R = X M + S Y, X and Y matrices of FP64
+// numbers brought to one unit (their larger exponent), M and S products of the
+// scaled links: E' = k' E from N and the links, R' = k'^3 R from E' and the pair
+// products.  Matrices whose numbers are not finite or outside the exponents' range
+// take FP64 instructions (force_two_fp64).  24^3 x 48: E 1.04 ms (2.81 with FP64
+// products, at the FP64 pipe's rate), R 2.82 ms (8.52).  Error of R on Gaussian
+// matrices and SU(3) links against exact sums: 6.3e-17 (FP64 sums 1.0e-16).
+
+// the limbs of a matrix in units of 2^(K - 1086), |entries| < 2^(K - 1028)
+__device__ __forceinline__ void f_limbs(const cd *v, int K, FixM3 &o)
+{
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        fix_limbs(fix_from_any(v[k].r, K), o.e[k].x, o.e[k].y);
+        fix_limbs(fix_from_any(v[k].i, K), o.e[k].z, o.e[k].w);
+    }
+}
+
+// the largest biased exponent of two matrices
+__device__ __forceinline__ int f_exponent(const cd *a, const cd *b)
+{
+    float m = 0.f;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        m = max3abs(m, __int_as_float(__double2hiint(a[k].r)), __int_as_float(__double2hiint(a[k].i)));
+        m = max3abs(m, __int_as_float(__double2hiint(b[k].r)), __int_as_float(__double2hiint(b[k].i)));
+    }
+    return __float_as_int(m) >> 20;
+}
+
+// X M + S Y with FP64 instructions, M and S from their limbs (exact to 2^-60)
+__device__ __noinline__ void force_two_fp64(const cd *X, const int4 *M, const int4 *S, int stride, const cd *Y, cd *R)
+{
+    auto value = [](int4 v) {
+        return cd{((double)v.x * 0x1p32 + (double)v.y) * 0x1p-60, ((double)v.z * 0x1p32 + (double)v.w) * 0x1p-60};
+    };
+    cd m[9], s[9];
+    for (int k = 0; k < 9; ++k) {
+        m[k] = value(M[k * stride]);
+        s[k] = value(S[k * stride]);
+    }
+    f_m3mul(X, m, R);
+    f_m3mul_acc(s, Y, R);
+}
+
+// R = X M + S Y, the limbs of M and S at [k stride]; bound: twelve products of a
+// 58-bit and a 60-bit number, middle sums below 12 (2^59 + 2^57) < 2^63
+__device__ __forceinline__ void force_two(const cd *X, const int4 *M, const int4 *S, int stride, const cd *Y, cd *R)
+{
+    const int e = f_exponent(X, Y);
+    if (e >= FIX_EMAX || (e < FIX_EMIN && e > 0)) {
+        cd x[9], y[9], r[9];
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+            x[k] = X[k];
+            y[k] = Y[k];
+        }
+        force_two_fp64(x, M, S, stride, y, r);
+#pragma unroll
+        for (int k = 0; k < 9; ++k) R[k] = r[k];
+        return;
+    }
+    constexpr int L = 5;
+    const int K = max(e, FIX_EMIN) + 6;
+    FixM3 fx, fy;
+    f_limbs(X, K, fx);
+    f_limbs(Y, K, fy);
+    const double sc = fix_pow2(K - 59 - L);  // hh's unit is 2^(K - 1082)
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            fix_t hr = 0, hi = 0, mr = 0x80000000LL >> L, mi = mr;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                fix_cmac(M[(k * 3 + j) * stride], fx.e[a * 3 + k], hr, mr, hi, mi);
+                fix_cmac(S[(a * 3 + k) * stride], fy.e[k * 3 + j], hr, mr, hi, mi);
+            }
+            R[a * 3 + j] = cd{sc * __ll2double_rn(fix_join_bits(hr, mr, L)), sc * __ll2double_rn(fix_join_bits(hi, mi, L))};
+        }
+}
+
+// k_force_E in fixed point: k' E_mu(x) and k' E_nu(x) of plane p
+__global__ void __launch_bounds__(128, 3) k_force_E_fix(Geom g, FixLinks U, const double2 *N, double2 *Eb)
+{
+    __shared__ int4 link[9 * 128];
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= g.V) return;
+    const int p = blockIdx.y;
+    const int mu = p < 3 ? 0 : (p < 5 ? 1 : 2);
+    const int nu = p < 3 ? p + 1 : (p < 5 ? p - 1 : 3);
+    int c[4];
+    site_coords(g, i, c);
+    const size_t V = (size_t)g.V;
+    int4 *const slot = link + threadIdx.x;  // read by this thread only
+#pragma unroll 1
+    for (int k = 0; k < 2; ++k) {
+        const int s0 = k == 0 ? 1 : 0, s1 = k == 0 ? 0 : 1;
+        const int4 *u = U.at(i, k == 0 ? mu : nu);
+#pragma unroll
+        for (int e = 0; e < 9; ++e) slot[e * 128] = __ldg(u + ((size_t)e << U.lvb));
+        cd X[9], Y[9], E[9];
+        f_N(N, g, c, mu, 0, nu, 0, p, X);
+        f_N(N, g, c, mu, s0, nu, s1, p, Y);
+        force_two(X, slot, slot, 128, Y, E);
+        double2 *o = Eb + (size_t)(p * 2 + k) * 9 * V + i;
+#pragma unroll
+        for (int e = 0; e < 9; ++e) o[e * V] = make_double2(E[e].r, E[e].i);
+    }
+}
+
+// k_force_plaq in fixed point: k'^3 R_A..R_D from k' E.  With the links in loop
+// order as 0..3 and P_n the product of links n and n + 1, R_n = E_{n+1} P_{n+2} +
+// P_{n+1} E_{n+3}.  The four P stay in shared memory (72 KB, three blocks per SM),
+// each thread its own.
+__global__ void __launch_bounds__(128, 3) k_force_plaq_fix(Geom g, FixLinks U, const double2 *Eb, double2 *Rb)
+{
+    extern __shared__ int4 prod[];  // [4][9][128]
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= g.V) return;
+    const int p = blockIdx.y;
+    const int mu = p < 3 ? 0 : (p < 5 ? 1 : 2);
+    const int nu = p < 3 ? p + 1 : (p < 5 ? p - 1 : 3);
+    int c[4];
+    site_coords(g, i, c);
+    const size_t V = (size_t)g.V;
+    int4 *const slot = prod + threadIdx.x;
+    int n[4] = {c[0], c[1], c[2], c[3]};
+    n[mu] = (n[mu] + 1) % g.L[mu];
+    const int xm = site_index(g, n);  // x + mu
+    n[mu] = c[mu];
+    n[nu] = (n[nu] + 1) % g.L[nu];
+    const int xn = site_index(g, n);  // x + nu
+    // link or E number k: A = U_mu(x), B = U_nu(x+mu), C = U_mu(x+nu)^+, D = U_nu(x)^+
+    auto site = [&](int k) { return k == 1 ? xm : (k == 2 ? xn : i); };
+#pragma unroll 1
+    for (int k = 0; k < 4; ++k) {
+        const int k1 = (k + 1) & 3;
+        FixM3 P, A;
+        P.load(U, site(k), k & 1 ? nu : mu, k >= 2);
+        A.load(U, site(k1), k1 & 1 ? nu : mu, k1 >= 2);
+        const fix_t half = 0x80000000LL >> 4;
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                fix_t hr = 0, hi = 0, mr = half, mi = half;
+#pragma unroll
+                for (int m = 0; m < 3; ++m) fix_cmac(A.e[m * 3 + j], P.e[a * 3 + m], hr, mr, hi, mi);
+                int4 o;
+                fix_limbs(fix_join_bits(hr, mr, 4), o.x, o.y);
+                fix_limbs(fix_join_bits(hi, mi, 4), o.z, o.w);
+                o.z = max(o.z, -0x7fffffff);
+                o.w = max(o.w, -0x7fffffff);
+                slot[(k * 9 + a * 3 + j) * 128] = o;
+            }
+    }
+    auto getE = [&](int k, cd *E) {
+        const double2 *q = Eb + (size_t)(p * 2 + (k & 1)) * 9 * V + site(k);
+        const bool dag = k >= 2;
+        const int sa = dag ? 1 : 3, sb = dag ? 3 : 1;
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+#pragma unroll
+            for (int b = 0; b < 3; ++b) {
+                const double2 v = q[(size_t)(a * sa + b * sb) * V];
+                E[a * 3 + b] = cd{v.x, __hiloint2double(__double2hiint(v.y) ^ (dag ? 0x80000000 : 0), __double2loint(v.y))};
+            }
+    };
+#pragma unroll 1
+    for (int k = 0; k < 4; ++k) {
+        cd X[9], Y[9], R[9];
+        getE((k + 1) & 3, X);
+        getE((k + 3) & 3, Y);
+        force_two(X, slot + ((k + 2) & 3) * 9 * 128, slot + ((k + 1) & 3) * 9 * 128, 128, Y, R);
+        double2 *o = Rb + (size_t)(p * 4 + k) * 9 * V + i;
+#pragma unroll
+        for (int e = 0; e < 9; ++e) o[e * V] = make_double2(R[e].r, R[e].i);
+    }
+}
+
 __device__ __forceinline__ int plane_of(int a, int b)
 {
     // (0,1) (0,2) (0,3) (1,2) (1,3) (2,3)
@@ -301,7 +485,7 @@ __device__ void hop_force(const Geom &g, const int c[4], int i, const Spinor64 &
 // plane (mu, s), s > mu, the link is A of the plaquette at x and C of the one
 // at x - s; in the plane (s, mu), s < mu, it is B of the plaquette at x - s
 // and D of the one at x.  Undaggered links take conj(c') R^+, daggered c' R.
-__global__ void k_force(Geom g, Gauge64 U, Spinor64 X, Spinor64 Y, const double2 *Rb, double kappa, double csw,
+__global__ void k_force(Geom g, Gauge64 U, Spinor64 X, Spinor64 Y, const double2 *Rb, double kappa, double kc,
                         double2 *out)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -316,9 +500,8 @@ __global__ void k_force(Geom g, Gauge64 U, Spinor64 X, Spinor64 Y, const double2
     else if (mu == 2) hop_force<2>(g, c, i, X, Y, kappa, G);
     else hop_force<3>(g, c, i, X, Y, kappa, G);
 
-    // c' = -i kc with kc = kappa c_SW / 4: conj(c') R^+ adds kc (Im, Re) of
-    // R's transpose, c' R adds kc (Im R, -Re R)
-    const double kc = kappa * csw / 4.0;
+    // c' = -i kc with kc = kappa c_SW / 4 (over k'^3 where R carries that factor):
+    // conj(c') R^+ adds kc (Im, Re) of R's transpose, c' R adds kc (Im R, -Re R)
     const size_t V = (size_t)g.V;
     auto get = [&](int p, int Xr, int site, cd *R) {
         const double2 *q = Rb + (size_t)(p * 4 + Xr) * 9 * V + site;
@@ -506,16 +689,31 @@ int force(mgc_clover_s *op, const double *phi, double *dSdU, const mgc_solve_par
     k_force_N<<<grid_for(g.V, 128), 128, 0, s>>>(g, Spinor64{X, g.lvb}, Spinor64{Y, g.lvb}, N);
     FCUDA(cudaGetLastError());
     count(1, (double)g.V * (2 * 192.0 + 54 * 16.0));
-    k_force_E<<<dim3(grid_for(g.V, 128), 6), 128, 0, s>>>(g, Gauge64{op->gauge->U64, g.lvb}, N, Eb);
+    const dim3 planes(grid_for(g.V, 128), 6);
+    double kc = op->kappa * op->csw / 4.0;
+    const FixLinks UQ{op->UQ, g.lvb};
+    if (op->CQ) {
+        const double ks = std::ldexp(op->kappa, -op->fix_ek);
+        kc /= ks * ks * ks;
+        k_force_E_fix<<<planes, 128, 0, s>>>(g, UQ, N, Eb);
+    } else {
+        k_force_E<<<planes, 128, 0, s>>>(g, Gauge64{op->gauge->U64, g.lvb}, N, Eb);
+    }
     FCUDA(cudaGetLastError());
     count(1, (double)g.V * (576.0 + 54 * 16.0 + 12 * 144.0));
-    k_force_plaq<<<dim3(grid_for(g.V, 128), 6), 128, 0, s>>>(g, Gauge64{op->gauge->U64, g.lvb}, Eb, Rb);
+    if (op->CQ) {
+        constexpr int smem = 4 * 9 * 128 * sizeof(int4);
+        FCUDA(cudaFuncSetAttribute(k_force_plaq_fix, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        k_force_plaq_fix<<<planes, 128, smem, s>>>(g, UQ, Eb, Rb);
+    } else {
+        k_force_plaq<<<planes, 128, 0, s>>>(g, Gauge64{op->gauge->U64, g.lvb}, Eb, Rb);
+    }
     FCUDA(cudaGetLastError());
     count(1, (double)g.V * (576.0 + 12 * 144.0 + 24 * 144.0));
     double2 *dst = p->on_device ? (double2 *)dSdU : gout;
     dim3 grid(grid_for(g.V, 128), 4);
     k_force<<<grid, 128, 0, s>>>(g, Gauge64{op->gauge->U64, g.lvb}, Spinor64{X, g.lvb}, Spinor64{Y, g.lvb}, Rb,
-                                 op->kappa, op->csw, dst);
+                                 op->kappa, kc, dst);
     FCUDA(cudaGetLastError());
     count(1, (double)g.V * (2 * 192.0 + 24 * 144.0 + 576.0));
     if (!p->on_device) FCUDA(cudaMemcpyAsync(dSdU, gout, gb, cudaMemcpyDeviceToHost, s));

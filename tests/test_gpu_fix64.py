@@ -191,3 +191,39 @@ def test_clover_build(name, kappa, csw, bent):
     cond = np.linalg.norm(ref, axis=(1, 2)) * np.linalg.norm(np.linalg.inv(ref), axis=(1, 2))
     err = np.linalg.norm(np.einsum("sij,sjk->sik", C, Ci) - np.eye(12), axis=(1, 2))
     assert (err < 6.7e-15 * cond * (cond if csw > 4 else 1.0)).all()
+
+
+@pytest.mark.parametrize("p", [-455, -400, 400, 470])
+def test_force_scales(p):
+    """dS/dU of 2^p phi is 2^(2p) times that of phi: the solves commute with powers of two, and the
+    matrix products do too but for the scales that run on FP64 instructions (p = -455: below 2^-894),
+    whose sums round differently: 1e-13."""
+    from paper_2112_00501_gb300 import api
+
+    name = "c4_8^4"
+    dims, block, eps, kappa, csw, U, phi = fields(name)
+    lat = api.Lattice(dims, block, -1)
+    op = api.CloverOperator(api.Gauge(lat, torch.from_numpy(U).cuda(), storage_prec=32), kappa, csw)
+    g0, _, _ = op.force(torch.from_numpy(phi).cuda())
+    g1, _, _ = op.force(torch.from_numpy(_scaled(phi, p)).cuda())
+    assert rel(_scaled(g1.cpu().numpy(), -2 * p), g0.cpu().numpy()) < 1e-13
+
+
+def test_force_links_without_fixed_point_copy():
+    """Bent links: the force's FP64 products, against the oracle's."""
+    from paper_2112_00501_gb300 import api
+
+    name = "c4_8^4"
+    dims, block, eps, kappa, csw, U, phi = fields(name)
+    U = U.copy()
+    U[5, 2] *= 1.01
+    lat = api.Lattice(dims, block, -1)
+    op = api.CloverOperator(api.Gauge(lat, torch.from_numpy(U).cuda(), storage_prec=32), kappa, csw)
+    g, _, _ = op.force(torch.from_numpy(phi).cuda())
+    Uf = U.copy()
+    Uf[5, 2] /= 1.01
+    opf = api.CloverOperator(api.Gauge(lat, torch.from_numpy(Uf).cuda(), storage_prec=32), kappa, csw)
+    gf, _, _ = opf.force(torch.from_numpy(phi).cuda())
+    # far from the bent link the two forces differ by its effect through the solves only
+    far = np.abs(np.arange(U.shape[0]) - 5) > U.shape[0] // 3
+    assert rel(g.cpu().numpy()[far], gf.cpu().numpy()[far]) < 1e-2

@@ -179,9 +179,12 @@ __global__ void __launch_bounds__(RT) k_map(long long n, F f)
     for (long long e = (long long)blockIdx.x * RT + threadIdx.x; e < n; e += (long long)gridDim.x * RT) f(e);
 }
 
+// One element per thread until the grid is full, so that small lattices use many
+// SMs: with four per thread a site pass over 8^4 ran in four blocks (42 us for the
+// correction sum, 28 us for the residual).
 static int red_grid(long long n)
 {
-    long long g = (n + RT * 4 - 1) / (RT * 4);
+    long long g = (n + RT - 1) / RT;
     if (g > RGRID_MAX) g = RGRID_MAX;
     if (g < 1) g = 1;
     return (int)g;
@@ -834,7 +837,8 @@ static int grid32(K kern, long long n4)
         while (per > 1 && sms * per > RGRID_MAX) --per;
         c = sms * per > RGRID_MAX ? RGRID_MAX : sms * per;
     }
-    long long need = (n4 + (long long)RT * U4 - 1) / ((long long)RT * U4);
+    // fewer than U4 entries per thread before fewer blocks than the device holds
+    long long need = (n4 + RT - 1) / RT;
     if (need < 1) need = 1;
     return need < c ? (int)need : c;
 }

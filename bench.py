@@ -985,6 +985,9 @@ def main():
                    "fp32_12real_gbs": by_d32 / t_d32 / 1e9, "fp32_us": 1e6 * t_d32,
                    "fp32_frac_hbm": (by_d32 / t_d32 / 1e9 / hbm) if hbm else None,
                    "fp64_gbs": by_d64 / t_d64 / 1e9, "fp64_us": 1e6 * t_d64,
+                   "fp64_frac_hbm": (by_d64 / t_d64 / 1e9 / hbm) if hbm else None,
+                   "fp64_note": "products on the integer multiply-add units (62-bit fixed point), so the "
+                                "conventional flops may exceed the FP64 FMA rate",
                    "fp16_frac_hbm": (by_d16 / t_d16 / 1e9 / hbm) if hbm else None,
                    "fp16_18real_gbs": by_d16_18 / t_d16_18 / 1e9, "fp16_18real_us": 1e6 * t_d16_18,
                    "fp16_18real_frac_hbm": (by_d16_18 / t_d16_18 / 1e9 / hbm) if hbm else None},

@@ -298,7 +298,7 @@ int launch_fix_clover(const Geom &g, const double2 *C64, int ek, int4 *out, int2
 
 // D, D^dagger at FP64 in block fixed point (fix64.cuh).  24^3 x 48: 372 us
 // against 1259 us with FP64 instructions (2.7 TB/s of compulsory bytes against
-// 0.8); the FMA pipe's heavy half, where the widening products run, is busy 67 %
+// 0.8); the FMA pipe's heavy half, where the widening products run, is busy 61 %
 // of the time.  Three blocks per SM (168 registers); four (128) spill 200 B per
 // thread and take 403 us.
 template <bool DAG, int LVB>

@@ -593,6 +593,69 @@ __global__ void __launch_bounds__(DIRAC_THREADS, (LVB > 0 && sizeof(typename SP:
     dst.store(i, psi);
 }
 
+// A at FP64 with the hopping sum in block fixed point, C^-1 with FP64 instructions:
+// 24^3 x 48 474 us against 1371 us with FP64 instructions throughout (error against
+// 64 bits 2.52e-16 and 2.59e-16); the FP64 pipe and the widening products share it.
+__device__ __noinline__ void apply_A_fp64(const Geom &g, int i, const Spinor64 &in, const Spinor64 &out,
+                                          const Gauge64 &U, const Clover64 &Ci, double kappa)
+{
+    int c[4];
+    site_coords(g, i, c);
+    Cx<double> acc[12], t[12], psi[12];
+    hop_site<false>(g, c, i, in, U, acc);
+    clover_site(Ci, i, acc, t);
+    in.load(i, psi);
+#pragma unroll
+    for (int k = 0; k < 12; ++k) psi[k] = Cx<double>{fma(-kappa, t[k].r, psi[k].r), fma(-kappa, t[k].i, psi[k].i)};
+    out.store(i, psi);
+}
+
+template <int LVB>
+__global__ void __launch_bounds__(FIX_THREADS, 3)
+    k_apply_A_fix(Geom g, Spinor64 in, Spinor64 out, FixLinks U, FixClover C, Gauge64 Ud, Clover64 Ci, double kappa)
+{
+    __shared__ int4 slots[(FIX_SPINOR_SLOTS + FIX_LINK_SLOTS) * FIX_THREADS];
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= g.V) return;
+    Spinor64 src = shift_rhs(in, blockIdx.y, g.V), dst = shift_rhs(out, blockIdx.y, g.V);
+    if (LVB > 0) {
+        g.lvb = LVB;
+#pragma unroll
+        for (int mu = 0; mu < 4; ++mu) g.lb[mu] = LVB / 4;
+        src.lvb = dst.lvb = U.lvb = Ci.lvb = LVB;
+    }
+    Cx<fix_t> acc[12];
+    int E;
+    if (!fix_dirac_sum<false, false>(g, i, src, U, C, slots + threadIdx.x, FIX_THREADS, acc, E)) {
+        apply_A_fp64(g, i, src, dst, Ud, Ci, kappa);
+        return;
+    }
+    const double sc = fix_pow2(E + C.ek - 55);
+    Cx<double> h[12], t[12], psi[12];
+#pragma unroll
+    for (int k = 0; k < 12; ++k) h[k] = Cx<double>{sc * __ll2double_rn(acc[k].r), sc * __ll2double_rn(acc[k].i)};
+    clover_site(Ci, i, h, t);
+    src.load(i, psi);
+#pragma unroll
+    for (int k = 0; k < 12; ++k) psi[k] = psi[k] - t[k];
+    dst.store(i, psi);
+}
+
+static void apply_A_fix(const mgc_clover_s *op, Spinor64 in, Spinor64 out, int nrhs, cudaStream_t s)
+{
+    const Geom &g = op->gauge->lat->g;
+    const bool cube = g.lb[0] == g.lb[1] && g.lb[1] == g.lb[2] && g.lb[2] == g.lb[3];
+    const dim3 grid(grid_for(g.V, FIX_THREADS), nrhs);
+    auto run = [&](auto kern) {
+        kern<<<grid, FIX_THREADS, 0, s>>>(g, in, out, FixLinks{op->UQ, g.lvb},
+                                          FixClover{op->CQ, op->CE, op->fix_ek, g.lvb}, Gauge64{op->gauge->U64, g.lvb},
+                                          Clover64{op->Ci64, g.lvb}, op->kappa);
+    };
+    if (cube && g.lvb == 8) run(k_apply_A_fix<8>);
+    else if (cube && g.lvb == 4) run(k_apply_A_fix<4>);
+    else run(k_apply_A_fix<0>);
+}
+
 template <class SP, class GA, class CL>
 static void apply_A_dispatch(const Geom &g, SP in, SP out, GA U, CL Ci, double kappa, int nrhs, cudaStream_t s)
 {
@@ -609,7 +672,9 @@ int launch_apply_A(const mgc_clover_s *op, int prec, const void *in, void *out, 
     const mgc_gauge_s *ga = op->gauge;
     const Geom &g = ga->lat->g;
     if (!has_prec(ga, prec)) return fail(MGC_ERR_INVALID_ARG, "no copy of the operator at this precision");
-    if (prec == 64) {
+    if (prec == 64 && op->CQ) {
+        apply_A_fix(op, sp64(g, in), sp64(g, out), nrhs, s);
+    } else if (prec == 64) {
         apply_A_dispatch(g, sp64(g, in), sp64(g, out), Gauge64{ga->U64, g.lvb}, Clover64{op->Ci64, g.lvb}, op->kappa,
                          nrhs, s);
     } else if (prec == 32) {

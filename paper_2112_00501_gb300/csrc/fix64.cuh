@@ -483,7 +483,8 @@ __device__ __noinline__ void fix_fallback(const Geom &g, int i, const Spinor64 &
 // instruction fetch for half its time (1060 us on 24^3 x 48).  The next hop's
 // spinor and link are copied to shared memory while this hop's products run;
 // without that, loads were the first stall (433 us).
-template <bool DAG>
+// CLOVER = false leaves the clover term out: kappa H psi = 2^(E + ek - 1078) acc.
+template <bool DAG, bool CLOVER = true>
 __device__ __forceinline__ bool fix_dirac_sum(const Geom &g, int i, const Spinor64 &in, const FixLinks &U,
                                               const FixClover &C, int4 *slots, int nt, Cx<fix_t> acc[12], int &E)
 {
@@ -508,7 +509,7 @@ __device__ __forceinline__ bool fix_dirac_sum(const Geom &g, int i, const Spinor
     fix_commit();
 
     int state = FIX_HOP;
-    {
+    if constexpr (CLOVER) {
         FixRaw r;
         r.load(in, i);
         r.range();
@@ -522,10 +523,14 @@ __device__ __forceinline__ bool fix_dirac_sum(const Geom &g, int i, const Spinor
 #pragma unroll
             for (int k = 0; k < 12; ++k) acc[k] = Cx<fix_t>{0, 0};
         }
-    }
-    // the sum is that of kappa H psi - C psi
+        // the sum is that of kappa H psi - C psi
 #pragma unroll
-    for (int k = 0; k < 12; ++k) acc[k] = -acc[k];
+        for (int k = 0; k < 12; ++k) acc[k] = -acc[k];
+    } else {
+        E = FIX_EMIN;
+#pragma unroll
+        for (int k = 0; k < 12; ++k) acc[k] = Cx<fix_t>{0, 0};
+    }
 #pragma unroll 1
     for (int d = 0; d < 8 && state != FIX_LEAVE; ++d) {
         const int m = (d & ~1) + (int)((bool)(d & 1) != DAG);

@@ -227,3 +227,23 @@ def test_force_links_without_fixed_point_copy():
     # far from the bent link the two forces differ by its effect through the solves only
     far = np.abs(np.arange(U.shape[0]) - 5) > U.shape[0] // 3
     assert rel(g.cpu().numpy()[far], gf.cpu().numpy()[far]) < 1e-2
+
+
+@pytest.mark.parametrize("name", ["c0_4^4", "ragged_8x4x12x8", "mid_8^4"])
+@pytest.mark.parametrize("kappa,kind", [(0.13, "plain"), (-0.2, "plain"), (0.13, "zeros"), (0.13, "point"),
+                                        (1e-6, "plain")])
+def test_apply_A(name, kappa, kind):
+    """A = C^-1 D; C^-1 on FP64 instructions adds a few of its roundings: 1e-15."""
+    dims, block, eps, _, csw, U, psi = fields(name)
+    psi = psi.copy()
+    if kind == "zeros":
+        psi[np.random.default_rng(3).random(psi.shape[0]) < 0.5] = 0
+    if kind == "point":
+        psi[:] = 0
+        psi[77, 2, 1] = 1.5 - 0.25j
+    two = np.stack([psi, np.roll(psi, 5, axis=0)])
+    got = _op(name, kappa=kappa).A(torch.from_numpy(two).cuda(), 64).cpu().numpy()
+    Cl = O.clover(dims, kappa, csw, U)
+    Ci = O.clover_inverse(dims, Cl)
+    for k in range(2):
+        assert rel(got[k], O.apply_A(dims, -1, kappa, U, Cl, Ci, two[k])) < 1e-15

@@ -195,8 +195,10 @@ __device__ __forceinline__ int2 fix_store(fix_t q)
 }
 
 // The links times ks (0 < |ks| < 1, as ks62 = ks 2^62) in units of 2^-60, rounded to
-// nearest; *bad is set unless the rows and columns of every link have norm 1 to
-// 1e-3, which bounds the operator's sums.
+// nearest; *bad is set unless every link is unitary to 1e-3 (norms of its rows and
+// columns, products of its rows), which bounds the operator's sums and those of the
+// links' products: with unit norms alone, four-link products could reach three
+// times a unitary field's, beyond the clover leaves' 64 bits.
 __global__ void k_fix_links(Geom g, Gauge64 U, long long ks62, int4 *__restrict__ out, int *bad)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -205,14 +207,23 @@ __global__ void k_fix_links(Geom g, Gauge64 U, long long ks62, int4 *__restrict_
     Cx<double> u[9];
     U.load(i, mu, u);
     int4 *o = out + (((size_t)(i >> g.lvb) * 4 + mu) * 9 << g.lvb) + (i & ((1 << g.lvb) - 1));
+    auto tofloat = [](Cx<double> z) { return Cx<float>{(float)z.r, (float)z.i}; };
     float n[9];
 #pragma unroll
-    for (int k = 0; k < 9; ++k) n[k] = norm2(Cx<float>{(float)u[k].r, (float)u[k].i});
+    for (int k = 0; k < 9; ++k) n[k] = norm2(tofloat(u[k]));
     bool fine = true;
 #pragma unroll
     for (int a = 0; a < 3; ++a)
         fine = fine && fabsf(n[3 * a] + n[3 * a + 1] + n[3 * a + 2] - 1.f) < 1e-3f &&
                fabsf(n[a] + n[3 + a] + n[6 + a] - 1.f) < 1e-3f;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const int b = a == 2 ? 0 : a + 1;
+        Cx<float> t = {0.f, 0.f};
+#pragma unroll
+        for (int k = 0; k < 3; ++k) t = cjfma(tofloat(u[3 * a + k]), tofloat(u[3 * b + k]), t);
+        fine = fine && norm2(t) < 1e-6f;
+    }
     if (!fine) atomicOr(bad, 1);
     auto scaled = [&](double x) {
         const long long q = fix_from_any(x, 1026) << 2;  // x 2^62, |x| < 1.001

@@ -99,6 +99,19 @@ def test_links_that_are_not_unitary():
     _check(name, fields(name)[6], U=U)
 
 
+@pytest.mark.parametrize("kappa", [0.12, 0.13])
+def test_links_with_dependent_rows(kappa):
+    """Rows and columns of norm 1 that are not orthogonal: no fixed-point copy.  C and D to the
+    FP64 path's roundings of a sum of 16 link products each up to 3 (1e-15 leaves a factor 4)."""
+    name = "mid_8^4"
+    dims, block, eps, _, csw, U, psi = fields(name)
+    r = np.random.default_rng(0)
+    J = np.exp(2j * np.pi * r.random((U.shape[0], 4, 1, 1))) * np.ones((3, 3)) / np.sqrt(3)
+    _check(name, psi, U=J, kappa=kappa, tol=1e-15)
+    C = _op(name, J, kappa).export_clover().cpu().numpy()
+    assert rel(C, O.clover(dims, kappa, csw, J).reshape(C.shape)) < 1e-15
+
+
 def test_batch_is_bit_identical():
     """A batch of one lattice with a fixed-point copy and one without."""
     from paper_2112_00501_gb300 import api

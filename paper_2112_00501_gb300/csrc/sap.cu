@@ -2286,9 +2286,9 @@ __global__ void __launch_bounds__(256, 1) k_sap_eo(Geom g, SP b, SP x, GA U, CL 
             pp = fmaf(w[k].r, w[k].r, fmaf(w[k].i, w[k].i, pp));
         }
         block_sum3(pr, pi, pp, red);
-        // a domain whose <p, p> is below FP32's normal range takes no step
-        const float ipp = pp >= FLT_MIN ? 1.0f / pp : 0.f;
-        const Cx<float> alpha = {pr * ipp, pi * ipp};
+        // quotients, not products with 1 / pp: small sources have pp below FP32's
+        // normal range, where its reciprocal overflows
+        const Cx<float> alpha = (pp > 0.f) ? Cx<float>{pr / pp, pi / pp} : Cx<float>{0.f, 0.f};
 #pragma unroll
         for (int k = 0; k < 6; ++k) {
             e[k] = cfma(alpha, rho[k], e[k]);

@@ -226,7 +226,7 @@ __global__ void k_fix_links(Geom g, Gauge64 U, long long ks62, int4 *__restrict_
     }
     if (!fine) atomicOr(bad, 1);
     auto scaled = [&](double x) {
-        const long long q = fix_from_any(x, 1026) << 2;  // x 2^62, |x| < 1.001
+        const long long q = fix_from_any(x, 1024);  // x 2^62, |x| < 1.001
         return fix_store(__mul64hi(q, ks62) + (long long)((unsigned long long)(q * ks62) >> 63));
     };
 #pragma unroll
@@ -307,17 +307,21 @@ int launch_fix_clover(const Geom &g, const double2 *C64, int ek, int4 *out, int2
     return MGC_OK;
 }
 
-// D, D^dagger at FP64 in block fixed point (fix64.cuh).  24^3 x 48: 372 us
-// against 1259 us with FP64 instructions (2.7 TB/s of compulsory bytes against
-// 0.8); the FMA pipe's heavy half, where the widening products run, is busy 61 %
-// of the time.  Three blocks per SM (168 registers); four (128) spill 200 B per
-// thread and take 403 us.
+// D, D^dagger at FP64 in block fixed point (fix64.cuh).  24^3 x 48: 393 us
+// against 1260 us with FP64 instructions (2.6 TB/s of compulsory bytes against
+// 0.8), 5 % of it the test of the components' sizes (372 us without); the FMA pipe's
+// heavy half, where the widening products run, is busy 61 % of the time without it.
+// Fields that leave fixed point at every site take 1273 us, fields that leave it at
+// some lanes of every warp up to both times (sites scaled at random by 2^-10 .. 2^10
+// 1440 us, by 2^-40 .. 2^40 1945 us).  Three blocks per SM (168 registers); four (128) spill 200 B per
+// thread and took 403 us against 372.
 template <bool DAG, int LVB>
 __global__ void __launch_bounds__(FIX_THREADS, 3)
     k_dirac_fix(Geom g, Spinor64 in, Spinor64 out, FixLinks U, FixClover C, Gauge64 Ud, Clover64 Cd, double kappa)
 {
-    __shared__ int4 slots[(FIX_SPINOR_SLOTS + FIX_LINK_SLOTS) * FIX_THREADS];
+    __shared__ int4 slots[FIX_SLOTS * FIX_THREADS];
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const unsigned lanes = __ballot_sync(0xffffffffu, i < g.V);
     if (i >= g.V) return;
     const int r = blockIdx.y;
     Spinor64 src = shift_rhs(in, r, g.V), dst = shift_rhs(out, r, g.V);
@@ -327,7 +331,9 @@ __global__ void __launch_bounds__(FIX_THREADS, 3)
         for (int mu = 0; mu < 4; ++mu) g.lb[mu] = LVB / 4;
         src.lvb = dst.lvb = U.lvb = C.lvb = LVB;
     }
-    if (!fix_dirac_site<DAG>(g, i, src, dst, U, C, slots + threadIdx.x)) fix_fallback<DAG>(g, i, src, dst, Ud, Cd, kappa);
+    const bool done = fix_dirac_site<DAG>(g, i, src, dst, U, C, slots + threadIdx.x);
+    __syncwarp(lanes);  // lanes leave at different hops: one FP64 pass for all of them
+    if (!done) fix_fallback<DAG>(g, i, src, dst, Ud, Cd, kappa);
 }
 
 template <int LVB>
@@ -605,7 +611,7 @@ __global__ void __launch_bounds__(DIRAC_THREADS, (LVB > 0 && sizeof(typename SP:
 }
 
 // A at FP64 with the hopping sum in block fixed point, C^-1 with FP64 instructions:
-// 24^3 x 48 474 us against 1371 us with FP64 instructions throughout (error against
+// 24^3 x 48 484 us against 1381 us with FP64 instructions throughout (error against
 // 64 bits 2.52e-16 and 2.59e-16); the FP64 pipe and the widening products share it.
 __device__ __noinline__ void apply_A_fp64(const Geom &g, int i, const Spinor64 &in, const Spinor64 &out,
                                           const Gauge64 &U, const Clover64 &Ci, double kappa)
@@ -625,8 +631,9 @@ template <int LVB>
 __global__ void __launch_bounds__(FIX_THREADS, 3)
     k_apply_A_fix(Geom g, Spinor64 in, Spinor64 out, FixLinks U, FixClover C, Gauge64 Ud, Clover64 Ci, double kappa)
 {
-    __shared__ int4 slots[(FIX_SPINOR_SLOTS + FIX_LINK_SLOTS) * FIX_THREADS];
+    __shared__ int4 slots[FIX_SLOTS * FIX_THREADS];
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const unsigned lanes = __ballot_sync(0xffffffffu, i < g.V);
     if (i >= g.V) return;
     Spinor64 src = shift_rhs(in, blockIdx.y, g.V), dst = shift_rhs(out, blockIdx.y, g.V);
     if (LVB > 0) {
@@ -636,8 +643,12 @@ __global__ void __launch_bounds__(FIX_THREADS, 3)
         src.lvb = dst.lvb = U.lvb = Ci.lvb = LVB;
     }
     Cx<fix_t> acc[12];
+    FixTerms terms;
     int E;
-    if (!fix_dirac_sum<false, false>(g, i, src, U, C, slots + threadIdx.x, FIX_THREADS, acc, E)) {
+    const bool done = fix_dirac_sum<false, false>(g, i, src, U, C, slots + threadIdx.x, FIX_THREADS, acc, terms, E) &&
+                      FixTotal(terms, slots + (FIX_SLOTS - 1) * FIX_THREADS + threadIdx.x).enough(terms.least(), acc);
+    __syncwarp(lanes);
+    if (!done) {
         apply_A_fp64(g, i, src, dst, Ud, Ci, kappa);
         return;
     }

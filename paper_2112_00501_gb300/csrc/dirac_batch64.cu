@@ -27,7 +27,7 @@ struct DiracBatchFix {
 template <bool DAG, int LVB>
 __global__ void __launch_bounds__(FIX_THREADS, 3) k_dirac_batch_fix(DiracBatchFix B)
 {
-    __shared__ int4 slots[(FIX_SPINOR_SLOTS + FIX_LINK_SLOTS) * FIX_THREADS];
+    __shared__ int4 slots[FIX_SLOTS * FIX_THREADS];
     int k = 0;
     while (k < B.n - 1 && (int)blockIdx.x >= B.end[k]) ++k;
     const int local = blockIdx.x - (k ? B.end[k - 1] : 0);
@@ -35,6 +35,7 @@ __global__ void __launch_bounds__(FIX_THREADS, 3) k_dirac_batch_fix(DiracBatchFi
     const int r = B.rhs_fast ? local % B.nrhs[k] : local / B.nsb[k];
     Geom g = B.g[k];
     const int i = sb * FIX_THREADS + threadIdx.x;
+    const unsigned lanes = __ballot_sync(0xffffffffu, i < g.V);
     if (i >= g.V) return;
     Spinor64 src = shift_rhs(B.in[k], r, g.V), dst = shift_rhs(B.out[k], r, g.V);
     FixLinks U = B.UQ[k];
@@ -45,7 +46,9 @@ __global__ void __launch_bounds__(FIX_THREADS, 3) k_dirac_batch_fix(DiracBatchFi
         for (int mu = 0; mu < 4; ++mu) g.lb[mu] = LVB / 4;
         src.lvb = dst.lvb = U.lvb = C.lvb = LVB;
     }
-    if (!C.p || !fix_dirac_site<DAG>(g, i, src, dst, U, C, slots + threadIdx.x))
+    const bool done = C.p && fix_dirac_site<DAG>(g, i, src, dst, U, C, slots + threadIdx.x);
+    __syncwarp(lanes);
+    if (!done)
         fix_fallback<DAG>(g, i, src, dst, B.U[k], B.C[k], B.kappa[k]);
 }
 

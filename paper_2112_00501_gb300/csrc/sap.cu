@@ -514,8 +514,22 @@ __global__ void __launch_bounds__(256, 2) k_sap_fix(Geom g, Spinor64 b, Spinor64
     Cx<double> rv[12];
     if (!x_zero) {
         Cx<fix_t> acc[12];
+        FixTerms terms;
         int E;
-        if (fix_dirac_sum<false>(g, i, xx, U, C, reinterpret_cast<int4 *>(smem) + l, vb, acc, E)) {
+        int4 *const slots = reinterpret_cast<int4 *>(smem) + l;
+        bool done = fix_dirac_sum<false>(g, i, xx, U, C, slots, vb, acc, terms, E);
+        const FixTotal total(terms, slots + (FIX_SLOTS - 1) * vb);
+        if (done && !total.all_reach(terms.least())) {
+            // b is a term of b - D x as well (high words order like the doubles)
+            const int b0 = __double2hiint(fix_pow2(E + C.ek - 55 + 48) * terms.least());
+#pragma unroll
+            for (int k = 0; k < 12; ++k) {
+                const double2 v = bb.at(i)[(size_t)k << b.lvb];
+                done = done && (total.of(k, acc[k]) >= terms.least() ||
+                                max(__double2hiint(v.x) & 0x7fffffff, __double2hiint(v.y) & 0x7fffffff) >= b0);
+            }
+        }
+        if (done) {
             const double sc = fix_pow2(E + C.ek - 55);
             bb.load(i, rv);
 #pragma unroll
@@ -572,6 +586,8 @@ __global__ void __launch_bounds__(256, 2) k_sap_fix(Geom g, Spinor64 b, Spinor64
                    eC.x, acc);
 #pragma unroll
         for (int k = 0; k < 12; ++k) acc[k] = -acc[k];
+        FixTerms terms;  // not used here
+        terms.clear();
 #pragma unroll 1
         for (int d = 0; d < 8; ++d) {
             const int mu = d >> 1;
@@ -592,7 +608,7 @@ __global__ void __launch_bounds__(256, 2) k_sap_fix(Geom g, Spinor64 b, Spinor64
                         return Cx<fix_t>{v.x, v.y};
                     },
                     d, back, h1, h0);
-                fix_hop(U.at(back ? blkbase | ln : i, mu), vb, d, back, h1, h0, acc);
+                fix_hop(U.at(back ? blkbase | ln : i, mu), vb, d, back, h1, h0, acc, terms);
             }
         }
         // inner products of p' and r' (the integers as doubles), then r' - beta p'

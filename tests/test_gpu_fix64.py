@@ -11,6 +11,7 @@ import pytest
 
 from helpers import fields, rel
 from oracle import oracle as O
+from paper_2112_00501_gb300 import synth
 
 pytestmark = pytest.mark.gpu
 
@@ -110,6 +111,44 @@ def test_links_with_dependent_rows(kappa):
     _check(name, psi, U=J, kappa=kappa, tol=1e-15)
     C = _op(name, J, kappa).export_clover().cpu().numpy()
     assert rel(C, O.clover(dims, kappa, csw, J).reshape(C.shape)) < 1e-15
+
+
+def _worst_component(a, b):
+    """The largest relative 2-norm error of a spin and colour over the lattice."""
+    return (np.linalg.norm(a - b, axis=0) / np.linalg.norm(b, axis=0)).max()
+
+
+def _graded(psi, axis, p):
+    """One colour (or one spin) of psi scaled by 2^-p."""
+    psi = psi.copy()
+    if axis == "colour":
+        psi[:, :, 2] *= 2.0**-p
+    else:
+        psi[:, 1] *= 2.0**-p
+    return psi
+
+
+@pytest.mark.parametrize("eps", [0.0, 1e-5, 0.02])
+@pytest.mark.parametrize("axis", ["colour", "spin"])
+def test_graded_components(eps, axis):
+    """Links that hardly mix the colours: every spin and colour of D, D^dagger and A, with the
+    operator's own C and C^-1, on its own.
+    A component's error in fixed point is 2^-53 of the terms that enter it where the site is accepted,
+    its rounding and the oracle's sum 1.5e-16 each: 4e-16; C^-1 adds a few roundings."""
+    name = "mid_8^4"
+    dims, block, _, kappa, csw, _, psi = fields(name)
+    U = synth.gauge_field(dims, eps, 41)
+    op = _op(name, U)
+    Cl = op.export_clover().cpu().numpy()
+    Ci = op.export_clover(inverse=True).cpu().numpy()
+    for p in (0, 1, 2, 3, 4, 5, 7, 10, 15, 20, 25, 40):
+        v = _graded(psi, axis, p)
+        x = torch.from_numpy(v).cuda()
+        for dagger in (False, True):
+            ref = O.dirac(dims, -1, kappa, U, Cl, v, dagger=dagger)
+            assert _worst_component(op.D(x, prec=64, dagger=dagger).cpu().numpy(), ref) < 4e-16, (p, dagger)
+        ref = O.apply_A(dims, -1, kappa, U, Cl, Ci, v)
+        assert _worst_component(op.A(x, 64).cpu().numpy(), ref) < 1e-15, p
 
 
 def test_batch_is_bit_identical():

@@ -307,9 +307,9 @@ int launch_fix_clover(const Geom &g, const double2 *C64, int ek, int4 *out, int2
     return MGC_OK;
 }
 
-// D, D^dagger at FP64 in block fixed point (fix64.cuh).  24^3 x 48: 393 us
-// against 1260 us with FP64 instructions (2.6 TB/s of compulsory bytes against
-// 0.8), 5 % of it the test of the components' sizes (372 us without); the FMA pipe's
+// D, D^dagger at FP64 in block fixed point (fix64.cuh).  24^3 x 48: 384 us
+// against 1260 us with FP64 instructions (2.7 TB/s of compulsory bytes against
+// 0.8), 3 % of it the test of the components' sizes (372 us without); the FMA pipe's
 // heavy half, where the widening products run, is busy 61 % of the time without it.
 // Fields that leave fixed point at every site take 1273 us, fields that leave it at
 // some lanes of every warp up to both times (sites scaled at random by 2^-10 .. 2^10
@@ -319,7 +319,7 @@ template <bool DAG, int LVB>
 __global__ void __launch_bounds__(FIX_THREADS, 3)
     k_dirac_fix(Geom g, Spinor64 in, Spinor64 out, FixLinks U, FixClover C, Gauge64 Ud, Clover64 Cd, double kappa)
 {
-    __shared__ int4 slots[FIX_SLOTS * FIX_THREADS];
+    __shared__ int4 slots[(FIX_SPINOR_SLOTS + FIX_LINK_SLOTS) * FIX_THREADS];
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const unsigned lanes = __ballot_sync(0xffffffffu, i < g.V);
     if (i >= g.V) return;
@@ -613,8 +613,7 @@ __global__ void __launch_bounds__(DIRAC_THREADS, (LVB > 0 && sizeof(typename SP:
 // A at FP64 with the hopping sum in block fixed point, C^-1 with FP64 instructions:
 // 24^3 x 48 484 us against 1381 us with FP64 instructions throughout (error against
 // 64 bits 2.52e-16 and 2.59e-16); the FP64 pipe and the widening products share it.
-__device__ __noinline__ void apply_A_fp64(const Geom &g, int i, const Spinor64 &in, const Spinor64 &out,
-                                          const Gauge64 &U, const Clover64 &Ci, double kappa)
+__device__ __noinline__ void apply_A_fp64(Geom g, int i, Spinor64 in, Spinor64 out, Gauge64 U, Clover64 Ci, double kappa)
 {
     int c[4];
     site_coords(g, i, c);
@@ -631,7 +630,7 @@ template <int LVB>
 __global__ void __launch_bounds__(FIX_THREADS, 3)
     k_apply_A_fix(Geom g, Spinor64 in, Spinor64 out, FixLinks U, FixClover C, Gauge64 Ud, Clover64 Ci, double kappa)
 {
-    __shared__ int4 slots[FIX_SLOTS * FIX_THREADS];
+    __shared__ int4 slots[(FIX_SPINOR_SLOTS + FIX_LINK_SLOTS) * FIX_THREADS];
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const unsigned lanes = __ballot_sync(0xffffffffu, i < g.V);
     if (i >= g.V) return;
@@ -646,7 +645,7 @@ __global__ void __launch_bounds__(FIX_THREADS, 3)
     FixTerms terms;
     int E;
     const bool done = fix_dirac_sum<false, false>(g, i, src, U, C, slots + threadIdx.x, FIX_THREADS, acc, terms, E) &&
-                      FixTotal(terms, slots + (FIX_SLOTS - 1) * FIX_THREADS + threadIdx.x).enough(terms.least(), acc);
+                      terms.enough(terms.least(), acc);
     __syncwarp(lanes);
     if (!done) {
         apply_A_fp64(g, i, src, dst, Ud, Ci, kappa);

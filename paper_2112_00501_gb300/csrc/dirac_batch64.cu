@@ -27,7 +27,7 @@ struct DiracBatchFix {
 template <bool DAG, int LVB>
 __global__ void __launch_bounds__(FIX_THREADS, 3) k_dirac_batch_fix(DiracBatchFix B)
 {
-    __shared__ int4 slots[FIX_SLOTS * FIX_THREADS];
+    __shared__ int4 slots[(FIX_SPINOR_SLOTS + FIX_LINK_SLOTS) * FIX_THREADS];
     int k = 0;
     while (k < B.n - 1 && (int)blockIdx.x >= B.end[k]) ++k;
     const int local = blockIdx.x - (k ? B.end[k - 1] : 0);

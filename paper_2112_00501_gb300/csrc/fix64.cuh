@@ -38,12 +38,12 @@
 // amplify) are a fixed number of units of 2^(E + ek - 56), 1.2 of them in the mean
 // square, whatever a component's size; FP64's error of a component goes with the
 // magnitudes of the terms that enter it.  So a site runs on fixed point only where
-// every one of its twelve components is large enough: FixTerms adds up the
-// magnitudes of the hops' contributions to each and of the sum itself (at most twice
-// the terms), which must reach 2^54 units.  Gaussian fields at kappa = 0.125 to
-// 0.1365, on links near and far from 1, c_SW 0 and 1, have 2^57.8 in the median and
-// 2^55.5 in the smallest of 4e5 components, so ordinary fields stay; a field whose
-// colours or spins differ by more than about 4 in scale without being mixed leaves.
+// every one of its twelve components is large enough: FixTerms adds up magnitudes of
+// the hops' contributions to it, which with the sum's own (together at most twice the
+// terms) must reach 2^54 units.  Gaussian fields at kappa = 0.125 to 0.1365, on links
+// near and far from 1, c_SW 0 and 1, have 2^57.5 in the median and no component of
+// 4e5 below 2^55, so ordinary fields stay; a field whose colours or spins differ by
+// more than about 4 in scale without being mixed leaves.
 // Measured for a colour scaled by 2^-p on unit links: its error is 1.4e-16 to
 // 1.6e-16 at every p from 0 to 50, as with FP64 instructions (1.5e-16); without the
 // test it was 1.1e-14 at p = 10.
@@ -63,10 +63,10 @@ constexpr int FIX_EMIN = 0x80;   // smallest biased exponent the fixed-point pat
 constexpr int FIX_EMAX = 0x7c0;  // first biased exponent it does not
 
 // threads of the operator's blocks, and the 16-byte staging slots a thread has in
-// shared memory (slot k of thread t at [k][t], NT threads): a neighbour's spinor,
-// a link, and counts set aside (FixTerms)
+// shared memory (slot k of thread t at [k][t], NT threads): a neighbour's spinor
+// and a link
 constexpr int FIX_THREADS = 128;
-constexpr int FIX_SPINOR_SLOTS = 12, FIX_LINK_SLOTS = 9, FIX_SLOTS = FIX_SPINOR_SLOTS + FIX_LINK_SLOTS + 1;
+constexpr int FIX_SPINOR_SLOTS = 12, FIX_LINK_SLOTS = 9;
 
 // 16-byte asynchronous copies global -> shared, read back by the thread that
 // issued them, so no barrier is involved
@@ -293,83 +293,48 @@ __device__ __forceinline__ void fix_project_limbs(Q q, int m, bool back, int h1[
     }
 }
 
-// Lower bounds of the terms that enter each of a site's twelve components: the
-// magnitudes |re| + |im| of the hops' contributions in counts of 2^48 units, per
-// colour a word with those of the upper spins 0 (low half) and 1.  A contribution is
-// at most 6.9 2^56 units, eight of them 2^61.8, so a count has 14 bits.  The lower
-// spins of the x and y hops take the contributions the other way round: half() puts
-// the counts of the hops 0 to 3 aside in a shared-memory slot of the thread, total()
-// adds them up.  That is three registers, which the smoother has none to spare of
-// (six cost its FP64 solve 18 % in spills), and 8 instructions a hop and colour.
+// Lower bounds of the terms that enter a site's components, in counts of 2^32 units:
+// per colour the sum over the hops of the smaller of the half spinor's two
+// contributions, |re| + |im|, which bounds those to each of the four spins whatever
+// the direction's spin map.  A contribution is at most 6.9 2^56 units, eight of them
+// 2^61.8.  (Counts per spin took six registers, which the smoother has none to spare
+// of: 18 % of its FP64 solve in spills.)
 struct FixTerms {
-    uint32_t n[3];
+    int n[3];
     int hops;
-    __device__ __forceinline__ void clear() { n[0] = n[1] = n[2] = 0, hops = 0; }
-    __device__ __forceinline__ void half(int4 *aside)
+    __device__ __forceinline__ void clear() { n[0] = n[1] = n[2] = hops = 0; }
+    // the unit grows by 2^d
+    __device__ __forceinline__ void shift(int d)
     {
-        *aside = make_int4(n[0], n[1], n[2], 0);
-        n[0] = n[1] = n[2] = 0;
-    }
-    // the unit grows by 2^d, d > 0; aside: the slot once half() has been called
-    __device__ __forceinline__ void shift(int d, int4 *aside)
-    {
-        const uint32_t keep = d < 16 ? (0xffffu >> d) * 0x10001u : 0u;
-        d &= 31;
 #pragma unroll
-        for (int a = 0; a < 3; ++a) n[a] = (n[a] >> d) & keep;
-        if (aside) {
-            const int4 v = *aside;
-            *aside = make_int4(((uint32_t)v.x >> d) & keep, ((uint32_t)v.y >> d) & keep, ((uint32_t)v.z >> d) & keep, 0);
-        }
+        for (int a = 0; a < 3; ++a) n[a] >>= min(d, 31);
     }
     static __device__ __forceinline__ uint32_t size(Cx<fix_t> v)
     {
         return (uint32_t)abs((int)(v.r >> 32)) + (uint32_t)abs((int)(v.i >> 32));
     }
-    // a hop's contribution to colour a
-    __device__ __forceinline__ void add(int a, Cx<fix_t> w0, Cx<fix_t> w1)
+    // a hop's contributions to colour a
+    __device__ __forceinline__ void add(int a, Cx<fix_t> w0, Cx<fix_t> w1) { n[a] += (int)min(size(w0), size(w1)); }
+    __device__ __forceinline__ bool all_reach(int least) const { return min(min(n[0], n[1]), n[2]) >= least; }
+    // component k of the sum, of value v, has `least` counts
+    __device__ __forceinline__ bool reaches(int least, int k, Cx<fix_t> v) const
     {
-        n[a] += __byte_perm(size(w0), size(w1), 0x7632);
+        return (uint32_t)n[k % 3] + size(v) >= (uint32_t)least;
     }
-    // the counts that every component needs: 2^54 units for eight hops (whose sum's
-    // error is 1.2 units), for fewer by the square root of their number
-    __device__ __forceinline__ int least() const { return hops > 4 ? 64 : (hops > 2 ? 45 : (hops > 1 ? 32 : 23)); }
-};
-
-// the counts of a site's components after its eight hops
-struct FixTotal {
-    uint32_t up[3], lo[3];
-    __device__ __forceinline__ FixTotal(const FixTerms &t, const int4 *aside)
-    {
-        const int4 v = *aside;
-        const uint32_t x[3] = {(uint32_t)v.x, (uint32_t)v.y, (uint32_t)v.z};
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            up[a] = t.n[a] + x[a];
-            lo[a] = t.n[a] + __byte_perm(x[a], 0, 0x1032);
-        }
-    }
-    __device__ __forceinline__ bool all_reach(int least) const
-    {
-        uint32_t v = __vminu2(up[0], lo[0]);
-#pragma unroll
-        for (int a = 1; a < 3; ++a) v = __vminu2(v, __vminu2(up[a], lo[a]));
-        return min(v & 0xffffu, v >> 16) >= least;
-    }
-    // counts of component k, its value v (in the same unit) included
-    __device__ __forceinline__ int of(int k, Cx<fix_t> v) const
-    {
-        const uint32_t t = (k < 6 ? up : lo)[k % 3];
-        return (int)(k / 3 & 1 ? t >> 16 : t & 0xffffu) + (int)(FixTerms::size(v) >> 16);
-    }
-    // whether the sum acc is good to FP64's precision in every component
+    // whether every component of the sum acc has `least` counts
     __device__ __forceinline__ bool enough(int least, const Cx<fix_t> acc[12]) const
     {
         if (all_reach(least)) return true;
         bool all = true;
 #pragma unroll
-        for (int k = 0; k < 12; ++k) all = all && of(k, acc[k]) >= least;
+        for (int k = 0; k < 12; ++k) all = all && reaches(least, k, acc[k]);
         return all;
+    }
+    // the counts that every component of the operator needs: 2^54 units for eight
+    // hops (whose sum's error is 1.2 units), for fewer by the square root of their number
+    __device__ __forceinline__ int least() const
+    {
+        return hops > 4 ? 1 << 22 : (hops > 2 ? 0x2d4000 : (hops > 1 ? 1 << 21 : 0x16a000));
     }
 };
 
@@ -378,7 +343,7 @@ struct FixTotal {
 // exceeds it; FIX_LEAVE when the site needs FP64.
 enum { FIX_LEAVE, FIX_ZERO, FIX_HOP };
 __device__ __forceinline__ int fix_half_spinor(const int4 *slot, int nt, int m, bool back, bool flip, Cx<fix_t> acc[12],
-                                                FixTerms &terms, int4 *aside, int &E, int h1[12], int h0[12])
+                                                FixTerms &terms, int &E, int h1[12], int h0[12])
 {
     FixRaw r;
     r.load_staged(slot, nt);
@@ -387,7 +352,7 @@ __device__ __forceinline__ int fix_half_spinor(const int4 *slot, int nt, int m, 
         const int d = min(r.emax - E, 62);
         const fix_t half = (fix_t)1 << (d - 1);
         E = r.emax;
-        terms.shift(d, aside);
+        terms.shift(d);
 #pragma unroll
         for (int k = 0; k < 12; ++k) acc[k] = Cx<fix_t>{(acc[k].r + half) >> d, (acc[k].i + half) >> d};
     }
@@ -558,8 +523,7 @@ __device__ __forceinline__ void fix_cmac(int4 u, int4 x, fix_t &hr, fix_t &mr, f
 
 // (D psi)(x) with FP64 instructions, for the sites the fixed-point path leaves
 template <bool DAG>
-__device__ __noinline__ void fix_fallback(const Geom &g, int i, const Spinor64 &in, const Spinor64 &out,
-                                          const Gauge64 &U, const Clover64 &C, double kappa)
+__device__ __noinline__ void fix_fallback(Geom g, int i, Spinor64 in, Spinor64 out, Gauge64 U, Clover64 C, double kappa)
 {
     int c[4];
     site_coords(g, i, c);
@@ -584,7 +548,6 @@ __device__ __forceinline__ bool fix_dirac_sum(const Geom &g, int i, const Spinor
                                               FixTerms &terms, int &E)
 {
     int4 *const ls = slots + FIX_SPINOR_SLOTS * nt;
-    int4 *const aside = ls + FIX_LINK_SLOTS * nt;
     auto copy_spinor = [&](int j) {
         const double2 *q = in.at(j);
 #pragma unroll
@@ -633,8 +596,7 @@ __device__ __forceinline__ bool fix_dirac_sum(const Geom &g, int i, const Spinor
         const int m = (d & ~1) + (int)((bool)(d & 1) != DAG);
         int h1[12], h0[12];
         fix_wait<1>();  // this hop's spinor (its link may be in flight)
-        if (d == 4) terms.half(aside);
-        state = fix_half_spinor(slots, nt, m, d & 1, flip, acc, terms, d < 4 ? nullptr : aside, E, h1, h0);
+        state = fix_half_spinor(slots, nt, m, d & 1, flip, acc, terms, E, h1, h0);
         if (d < 7) {
             // every slot has been read: the test above depends on all of them
             j = fix_neighbour(g, c, d + 1, flip);
@@ -665,7 +627,7 @@ __device__ __forceinline__ bool fix_dirac_site(const Geom &g, int i, const Spino
     FixTerms terms;
     int E;
     if (!fix_dirac_sum<DAG>(g, i, in, U, C, slots, FIX_THREADS, acc, terms, E)) return false;
-    if (!FixTotal(terms, slots + (FIX_SLOTS - 1) * FIX_THREADS).enough(terms.least(), acc)) return false;
+    if (!terms.enough(terms.least(), acc)) return false;
     const double sc = -fix_pow2(E + C.ek - 55);
     Cx<double> o[12];
 #pragma unroll

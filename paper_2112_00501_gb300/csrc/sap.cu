@@ -365,13 +365,15 @@ __global__ void __launch_bounds__(256) k_sap_colour(Geom g, SP b, SP x, GA U, CL
 // are FP64 as before, on the integers' doubles r' and p': with
 // beta = <p', r'>/<p', p'>, alpha = -beta 2^(-4 - ek) and r - alpha p is
 // 2^(E - 1082) (r' - beta p').  A domain whose residual is not finite or outside
-// 2^-894 .. 2^961 runs on FP64 instructions (mr_domain_fp64).
+// 2^-894 .. 2^961, or one where a component of D_B r is too small for the unit at
+// any step (SAP_FIX_LEAST), is solved with FP64 instructions instead
+// (sap_domain_fp64); at a site of the residual the source b counts as a term too.
 //
 // Bound: FP64 pipe (56 % busy; conversions, inner products and updates) and the
 // widening products in turn.  r and e in shared memory (98 KB) and 128 registers
 // give two blocks per SM; the residual's staging slots lie over r and e, which
-// come later.  16^3 x 32, 4 steps: 281 us a colour against 883 us with FP64
-// instructions.  Error of two sweeps against quadruple precision on 8^4: 1.0e-16
+// come later.  16^3 x 32, 4 steps from a guess: 373 us a colour (356 us without the
+// tests of the components' sizes) against 910 us with FP64 instructions.  Error of two sweeps against quadruple precision on 8^4: 1.0e-16
 // against 2.3e-16.
 
 // the largest biased exponent of 24 reals
@@ -407,8 +409,9 @@ __device__ __forceinline__ double two_sum(double s, double t, double &err)
 // alpha = (pr + i pi)/pp of the block's sums: block_sum3 with the warps' partials
 // added pairwise in double-double by the lanes of each warp, and quotients with
 // their remainders, so that alpha's error (which every component of e shares) is
-// little more than its own rounding.  A zero pp gives zero.
-__device__ __forceinline__ Cx<double> block_alpha(double pr, double pi, double pp, double *red)
+// little more than its own rounding.  A zero pp gives zero.  small becomes true on
+// every thread where it is on one.
+__device__ __forceinline__ Cx<double> block_alpha(double pr, double pi, double pp, double *red, bool &small)
 {
     const int nt = blockDim.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const unsigned mask = nt >= 32 ? 0xffffffffu : ((1u << nt) - 1u);
@@ -422,7 +425,7 @@ __device__ __forceinline__ Cx<double> block_alpha(double pr, double pi, double p
     double prl = 0, pil = 0, ppl = 0;
     if (nt > 32) {
         if (lane < 3) red[(lane << 3) + warp] = lane == 0 ? pr : (lane == 1 ? pi : pp);
-        __syncthreads();
+        small = __syncthreads_or(small);
         // lane 8 v + w holds warp w's partial of value v (at most eight warps)
         double s = lane < 24 && (lane & 7) < (nt >> 5) ? red[lane] : 0.0, lo = 0;
 #pragma unroll
@@ -439,7 +442,7 @@ __device__ __forceinline__ Cx<double> block_alpha(double pr, double pi, double p
         pil = __shfl_sync(mask, lo, 8);
         ppl = __shfl_sync(mask, lo, 16);
     } else {
-        __syncthreads();
+        small = __syncthreads_or(small);
     }
     if (!(pp > 0)) return Cx<double>{0, 0};
     const double inv = 1.0 / pp;
@@ -448,11 +451,21 @@ __device__ __forceinline__ Cx<double> block_alpha(double pr, double pi, double p
                       fma(fma(-qi, pp, pi) + fma(-qi, ppl, pil), inv, qi)};
 }
 
-__device__ __noinline__ void mr_domain_fp64(const Gauge64 &U, const Clover64 &C, double kappa, int blkbase, int i,
-                                            int l, int vb, const Geom &g, const int *lc, Cx<double> *rs, double *red,
-                                            int nmr, Cx<double> *rv, Cx<double> *e)
+__device__ __noinline__ void dirac_site_fp64(Geom g, int i, Spinor64 x, Gauge64 U, Clover64 C, double kappa,
+                                             Cx<double> *out)
 {
-    int nf[4], nb[4];
+    int c[4];
+    site_coords(g, i, c);
+    dirac_site<false>(g, c, i, x, U, C, kappa, out);
+}
+
+// a domain's residual, MR and update with FP64 instructions
+__device__ __noinline__ void sap_domain_fp64(Geom g, int blkbase, int l, Spinor64 b, Spinor64 x, Gauge64 U, Clover64 C,
+                                             double kappa, Cx<double> *rs, double *red, int nmr, int x_zero)
+{
+    const int vb = 1 << g.lvb, i = blkbase | l;
+    int lc[4], nf[4], nb[4];
+    local_coords(g, l, lc);
 #pragma unroll
     for (int mu = 0; mu < 4; ++mu) {
         int t[4] = {lc[0], lc[1], lc[2], lc[3]};
@@ -461,21 +474,37 @@ __device__ __noinline__ void mr_domain_fp64(const Gauge64 &U, const Clover64 &C,
         t[mu] = lc[mu] - 1;
         nb[mu] = (t[mu] >= 0) ? local_index(g, t) : -1;
     }
+    Cx<double> r[12], e[12];
+    b.load(i, r);
+    if (!x_zero) {
+        Cx<double> dx[12];
+        dirac_site_fp64(g, i, x, U, C, kappa, dx);
 #pragma unroll
-    for (int k = 0; k < 12; ++k) rs[k * vb + l] = rv[k];
+        for (int k = 0; k < 12; ++k) r[k] = r[k] - dx[k];
+    }
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+        e[k] = Cx<double>{0, 0};
+        rs[k * vb + l] = r[k];
+    }
     __syncthreads();
-    mr_domain(U, C, kappa, blkbase, i, l, vb, nf, nb, rs, red, nmr, rv, e);
-}
-
-__device__ __noinline__ void dirac_site_fp64(const Geom &g, int i, const Spinor64 &x, const Gauge64 &U,
-                                             const Clover64 &C, double kappa, Cx<double> *out)
-{
-    int c[4];
-    site_coords(g, i, c);
-    dirac_site<false>(g, c, i, x, U, C, kappa, out);
+    mr_domain(U, C, kappa, blkbase, i, l, vb, nf, nb, rs, red, nmr, r, e);
+    if (!x_zero) {
+        Cx<double> xo[12];
+        x.load(i, xo);
+#pragma unroll
+        for (int k = 0; k < 12; ++k) e[k] = e[k] + xo[k];
+    }
+    x.store(i, e);
 }
 
 constexpr size_t sap_fix_smem(int vb) { return (size_t)vb * 24 * 16 + 96 * sizeof(double) + 32 * sizeof(int); }
+
+// The counts (FixTerms) that every component of D_B r needs: 2^52 units.  The unit
+// is the whole domain's here and corner sites have four hops, so that Gaussian
+// residuals reach down to 2^53.5 (4e5 components, four steps; median 2^56.8); at
+// 2^53 one domain in 10^4 would leave, each holding its launch up by 300 us.
+constexpr int SAP_FIX_LEAST = 1 << (52 - 32);
 
 template <int LVB>
 __global__ void __launch_bounds__(256, 2) k_sap_fix(Geom g, Spinor64 b, Spinor64 x, FixLinks U, FixClover C, Gauge64 Ud,
@@ -516,16 +545,14 @@ __global__ void __launch_bounds__(256, 2) k_sap_fix(Geom g, Spinor64 b, Spinor64
         Cx<fix_t> acc[12];
         FixTerms terms;
         int E;
-        int4 *const slots = reinterpret_cast<int4 *>(smem) + l;
-        bool done = fix_dirac_sum<false>(g, i, xx, U, C, slots, vb, acc, terms, E);
-        const FixTotal total(terms, slots + (FIX_SLOTS - 1) * vb);
-        if (done && !total.all_reach(terms.least())) {
+        bool done = fix_dirac_sum<false>(g, i, xx, U, C, reinterpret_cast<int4 *>(smem) + l, vb, acc, terms, E);
+        if (done && !terms.all_reach(terms.least())) {
             // b is a term of b - D x as well (high words order like the doubles)
-            const int b0 = __double2hiint(fix_pow2(E + C.ek - 55 + 48) * terms.least());
+            const int b0 = __double2hiint(fix_pow2(E + C.ek - 55 + 32) * terms.least());
 #pragma unroll
             for (int k = 0; k < 12; ++k) {
                 const double2 v = bb.at(i)[(size_t)k << b.lvb];
-                done = done && (total.of(k, acc[k]) >= terms.least() ||
+                done = done && (terms.reaches(terms.least(), k, acc[k]) ||
                                 max(__double2hiint(v.x) & 0x7fffffff, __double2hiint(v.y) & 0x7fffffff) >= b0);
             }
         }
@@ -547,31 +574,17 @@ __global__ void __launch_bounds__(256, 2) k_sap_fix(Geom g, Spinor64 b, Spinor64
         bb.load(i, rv);
     }
     const int e0 = block_max(fix_exponent(rv), redi);  // a barrier: the staging slots are free
-    if (e0 >= FIX_EMAX || (e0 < FIX_EMIN && e0 > 0)) {
-        Cx<double> r[12], e[12];
-#pragma unroll
-        for (int k = 0; k < 12; ++k) {
-            r[k] = rv[k];
-            e[k] = Cx<double>{0, 0};
-        }
-        mr_domain_fp64(Ud, Cd, kappa, blkbase, i, l, vb, g, lc, reinterpret_cast<Cx<double> *>(smem), red, nmr, r, e);
-        if (!x_zero) {
-            Cx<double> xo[12];
-            xx.load(i, xo);
-#pragma unroll
-            for (int k = 0; k < 12; ++k) e[k] = e[k] + xo[k];
-        }
-        xx.store(i, e);
-        return;
-    }
+    bool fp64 = e0 >= FIX_EMAX || (e0 < FIX_EMIN && e0 > 0);
 
-    // 2. minimal residual
+    // 2. minimal residual; e holds r until the first step, whose alpha r takes r's
+    // doubles (the integers drop what lies below 2^-60 of the domain's largest)
 #pragma unroll
-    for (int k = 0; k < 12; ++k) es[k * vb + l] = make_double2(0.0, 0.0);
+    for (int k = 0; k < 12; ++k) es[k * vb + l] = make_double2(rv[k].r, rv[k].i);
     const int2 eC = __ldg(C.e + i);
     int E = e0 + dE, K = e0 + dE + 4;
+    int it = 0;
 #pragma unroll 1
-    for (int it = 0; it < nmr && E > FIX_EMIN / 2 + 32 + dE; ++it) {
+    for (; !fp64 && it < nmr && E > FIX_EMIN / 2 + 32 + dE; ++it) {
         // r in the domain's unit (a zero residual has e0 = 0 and no step)
 #pragma unroll
         for (int k = 0; k < 12; ++k)
@@ -586,7 +599,7 @@ __global__ void __launch_bounds__(256, 2) k_sap_fix(Geom g, Spinor64 b, Spinor64
                    eC.x, acc);
 #pragma unroll
         for (int k = 0; k < 12; ++k) acc[k] = -acc[k];
-        FixTerms terms;  // not used here
+        FixTerms terms;
         terms.clear();
 #pragma unroll 1
         for (int d = 0; d < 8; ++d) {
@@ -611,6 +624,7 @@ __global__ void __launch_bounds__(256, 2) k_sap_fix(Geom g, Spinor64 b, Spinor64
                 fix_hop(U.at(back ? blkbase | ln : i, mu), vb, d, back, h1, h0, acc, terms);
             }
         }
+        fp64 = !terms.enough(SAP_FIX_LEAST, acc);
         // inner products of p' and r' (the integers as doubles), then r' - beta p'
         double pr = 0, pi = 0, pp = 0;
         Cx<double> p[12];
@@ -623,16 +637,31 @@ __global__ void __launch_bounds__(256, 2) k_sap_fix(Geom g, Spinor64 b, Spinor64
             pi = fma(p[k].r, ri, fma(-p[k].i, rr, pi));
             pp = fma(p[k].r, p[k].r, fma(p[k].i, p[k].i, pp));
         }
-        const Cx<double> beta = block_alpha(pr, pi, pp, red);
-        const Cx<double> a = -fix_pow2(E - 63 - C.ek) * beta;  // r = 2^(E - 1082) r', alpha = -beta 2^(-4 - ek)
+        const Cx<double> beta = block_alpha(pr, pi, pp, red, fp64);
+        if (fp64) break;
+        // alpha = -beta 2^(-4 - ek) on r, the more 2^(E - 1082) on r'
+        const Cx<double> a = -fix_pow2(it == 0 ? 1019 - C.ek : E - 63 - C.ek) * beta;
 #pragma unroll
         for (int k = 0; k < 12; ++k) {
             const longlong2 v = rs[k * vb + l];
             const Cx<double> r = {__ll2double_rn(v.x), __ll2double_rn(v.y)};
-            const double2 e = es[k * vb + l];
-            const Cx<double> en = cfma(a, r, Cx<double>{e.x, e.y});
-            es[k * vb + l] = make_double2(en.r, en.i);
             rv[k] = r - beta * p[k];
+        }
+        if (it == 0) {
+#pragma unroll
+            for (int k = 0; k < 12; ++k) {
+                const double2 e = es[k * vb + l];
+                const Cx<double> en = a * Cx<double>{e.x, e.y};
+                es[k * vb + l] = make_double2(en.r, en.i);
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < 12; ++k) {
+                const longlong2 v = rs[k * vb + l];
+                const double2 e = es[k * vb + l];
+                const Cx<double> en = cfma(a, Cx<double>{__ll2double_rn(v.x), __ll2double_rn(v.y)}, Cx<double>{e.x, e.y});
+                es[k * vb + l] = make_double2(en.r, en.i);
+            }
         }
         if (it + 1 < nmr) {
             // rv is in units of 2^(E - 1082); a zero residual ends the loop
@@ -642,12 +671,17 @@ __global__ void __launch_bounds__(256, 2) k_sap_fix(Geom g, Spinor64 b, Spinor64
         }
     }
 
+    if (fp64) {
+        sap_domain_fp64(g, blkbase, l, bb, xx, Ud, Cd, kappa, reinterpret_cast<Cx<double> *>(smem), red, nmr, x_zero);
+        return;
+    }
+
     // 3. x_B += e
     Cx<double> e[12];
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
         const double2 v = es[k * vb + l];
-        e[k] = Cx<double>{v.x, v.y};
+        e[k] = it > 0 ? Cx<double>{v.x, v.y} : Cx<double>{0, 0};
     }
     if (!x_zero) {
         Cx<double> xo[12];
@@ -2378,10 +2412,10 @@ static int sap_run(const Geom &g, SP b, SP x, GA U, CL C, CL Ci, double kappa, i
     return MGC_OK;
 }
 
-// The largest room the fixed-point MR leaves for the clover term: beyond it
-// (kappa below about 1/1000) r would keep less than FP64's 53 bits below the
-// domain's largest component.
-constexpr int SAP_FIX_MAX_ROOM = 6;
+// The largest room the fixed-point MR leaves for the clover term: beyond it (kappa
+// below about 1/250) the hops are so small in the domain's unit that most domains
+// would find a component too small (SAP_FIX_LEAST) and run on FP64 after all.
+constexpr int SAP_FIX_MAX_ROOM = 3;
 
 template <int LVB>
 static int sap_run_fix(const mgc_clover_s *op, const void *b, void *x, int nrhs, int n_cy, int n_mr, int x_is_zero,

@@ -214,6 +214,25 @@ def test_sap_sparse_and_zero_domains():
     _check_sap(name, b)
 
 
+@pytest.mark.parametrize("eps", [0.0, 1e-5])
+@pytest.mark.parametrize("axis", ["colour", "spin"])
+@pytest.mark.parametrize("n_cy,n_mr", [(1, 1), (2, 4)])
+def test_sap_graded_components(eps, axis, n_cy, n_mr):
+    """As test_graded_components, for the smoother.  Every component carries alpha's error: the oracle
+    adds a domain's N = 3072 products one after another, a random walk of sqrt(N) u = 6e-15 in <p, r>
+    and in <p, p>, together 9e-15.  (Without a test of the sizes a colour at 2^-20 was off by 2e-11.)"""
+    name = "mid_8^4"
+    dims, block, _, kappa, csw, _, psi = fields(name)
+    U = synth.gauge_field(dims, eps, 41)
+    op = _op(name, U)
+    Cl = op.export_clover().cpu().numpy()
+    for p in (0, 1, 2, 3, 4, 5, 7, 10, 15, 20, 25, 40, 60):
+        b = _graded(psi, axis, p)
+        got = op.sap(torch.from_numpy(b).cuda(), 64, n_cy, n_mr).cpu().numpy()
+        ref = O.sap(dims, block, -1, kappa, U, Cl, b, ncy=n_cy, nmr=n_mr)
+        assert _worst_component(got, ref) < 1e-14, p
+
+
 def test_sap_non_finite():
     b = fields("mid_8^4")[6].copy()
     b[100, 1, 2] = np.nan

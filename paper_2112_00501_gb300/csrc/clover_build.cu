@@ -179,8 +179,8 @@ __global__ void k_clover_build(Geom g, Gauge64 U, double kappa, double csw, doub
 
 // ---- the build from the fixed-point links (fix64.cuh): the leaves' matrix
 // products on the integer multiply-add units, one thread per site and plane, then
-// C and C^-1 per site with FP64 instructions.  24^3 x 48: 2.1 and 2.3 ms, against
-// 19.1 ms with FP64 products, a generic sigma table and Gauss-Jordan elimination
+// C and C^-1 per site with FP64 instructions.  24^3 x 48: 2.2 and 2.3 ms (leaves of
+// weak fields, which run on FP64 instructions, 8.8 ms), against 19.1 ms with FP64 products, a generic sigma table and Gauss-Jordan elimination
 // throughout, bound by the FP64 pipe.  Error of C^-1 against quadruple precision:
 // 9.4e-17 (1.5e-16 by elimination).
 
@@ -210,11 +210,64 @@ __device__ __forceinline__ void fix_row_mul(const int4 p[3], const FixM3 &A, int
     }
 }
 
+// The magnitudes of the terms of the nine reals of Q - Q^+ (below) in the product
+// P A, added to S in units of 2^-56 of the scaled links
+__device__ __forceinline__ void leaf_terms(const FixM3 &P, const FixM3 &A, float *S, int stride)
+{
+    auto mag = [](int hi) { return (float)abs(hi); };
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            float re = 0.f, im = 0.f;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const float pr = mag(P.e[3 * a + k].x), pi = mag(P.e[3 * a + k].z);
+                const float ar = mag(A.e[3 * k + b].x), ai = mag(A.e[3 * k + b].z);
+                if (a != b) re = fmaf(pr, ar, fmaf(pi, ai, re));
+                im = fmaf(pr, ai, fmaf(pi, ar, im));
+            }
+            if (a == b) {
+                S[a * stride] += 2.f * im;
+            } else {
+                const int hi = a > b ? a : b, lo = a > b ? b : a, o = 3 + 2 * (hi - 1 + lo);
+                S[o * stride] += re;
+                S[(o + 1) * stride] += im;
+            }
+        }
+}
+
+// The same nine reals with FP64 instructions from the links themselves, scale =
+// 2^59 k'^4
+__device__ __noinline__ void leaves_fp64(Geom g, Gauge64 U, int x, int mu, int nu, double scale, double *G)
+{
+    int c[4];
+    site_coords(g, x, c);
+    cd Q[9];
+    clover_leaves(g, U, c, x, mu, nu, Q);
+    for (int k = 0; k < 3; ++k) G[k] = scale * (2 * Q[4 * k].i);
+    int o = 3;
+    for (int a = 1; a < 3; ++a)
+        for (int b = 0; b < a; ++b) {
+            G[o++] = scale * (Q[3 * a + b].r - Q[3 * b + a].r);
+            G[o++] = scale * (Q[3 * a + b].i + Q[3 * b + a].i);
+        }
+}
+
 // Q - Q^+ of plane blockIdx.y at every site, Q the sum of its four leaves of the
 // scaled links: three imaginary diagonals and the entries (1,0), (2,0), (2,1), nine
-// reals in units of 2^-59, to F as reals 9 plane + k of a packed clover term
-__global__ void __launch_bounds__(128, 4) k_clover_leaves(Geom g, FixLinks U, double *F, const int *no_fix)
+// reals in units of 2^-59, to F as reals 9 plane + k of a packed clover term.
+// Their error is some units whatever their size, with FP64 instructions it goes with
+// the terms' magnitudes: fields exp(i eps H) have the same error, 2.6e-16 of the
+// off-diagonal reals, at eps = 0.11.  A site and plane with a real whose terms (those
+// of the last products, leaf_terms) stay below LEAF_LEAST, which such fields do and
+// fields of eps >= 0.3 do not (smallest of 1.5e5 reals 2^55.4; k' = 1/2, the worst),
+// is computed with FP64 instructions.
+constexpr float LEAF_LEAST = 0x1p52f;  // 2^55 units
+__global__ void __launch_bounds__(128, 4) k_clover_leaves(Geom g, FixLinks U, Gauge64 Ud, double scale, double *F,
+                                                          const int *no_fix)
 {
+    __shared__ float terms[9 * 128];
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= g.V || *no_fix) return;
     const int p = blockIdx.y;
@@ -223,8 +276,12 @@ __global__ void __launch_bounds__(128, 4) k_clover_leaves(Geom g, FixLinks U, do
     int c[4];
     site_coords(g, x, c);
     fix_t G[9];
+    float *const S = terms + threadIdx.x;  // this thread's
 #pragma unroll
-    for (int k = 0; k < 9; ++k) G[k] = 0;
+    for (int k = 0; k < 9; ++k) {
+        G[k] = 0;
+        S[k * 128] = 0.f;
+    }
 #pragma unroll 1
     for (int leaf = 0; leaf < 4; ++leaf) {
         FixM3 P;
@@ -245,6 +302,7 @@ __global__ void __launch_bounds__(128, 4) k_clover_leaves(Geom g, FixLinks U, do
             }
             FixM3 A;
             A.load(U, site, dir, w.dag);
+            if (step == 3) leaf_terms(P, A, S, 128);
             Cx<fix_t> r[9];
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
@@ -272,10 +330,20 @@ __global__ void __launch_bounds__(128, 4) k_clover_leaves(Geom g, FixLinks U, do
         }
     }
     double *o = F + 2 * (((size_t)(x >> g.lvb) * 36 << g.lvb) + (x & ((1 << g.lvb) - 1)));
-#pragma unroll
-    for (int k = 0; k < 9; ++k) {
+    auto put = [&](int k, double v) {
         const int r = 9 * p + k;
-        o[((size_t)(r >> 1) << (g.lvb + 1)) + (r & 1)] = __ll2double_rn(G[k]);
+        o[((size_t)(r >> 1) << (g.lvb + 1)) + (r & 1)] = v;
+    };
+    bool fine = true;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) fine = fine && S[k * 128] >= LEAF_LEAST;
+    if (fine) {
+#pragma unroll
+        for (int k = 0; k < 9; ++k) put(k, __ll2double_rn(G[k]));
+    } else {
+        double D[9];
+        leaves_fp64(g, Ud, x, mu, nu, scale, D);
+        for (int k = 0; k < 9; ++k) put(k, D[k]);
     }
 }
 
@@ -496,9 +564,10 @@ int launch_clover_build(const Geom &g, const double2 *U64, const int4 *UQ, doubl
                         double csw, double2 *C64, double2 *Ci64, int *d_bad, cudaStream_t s)
 {
     if (UQ) {
-        k_clover_leaves<<<dim3(grid_for(g.V, 128), 6), 128, 0, s>>>(g, FixLinks{UQ, g.lvb}, (double *)Ci64, no_fix);
-        k_clover_assemble<<<grid_for(g.V, 128), 128, 0, s>>>(g, kappa * csw * 0x1p-62 / (ks * ks * ks * ks), C64, Ci64,
-                                                             d_bad, no_fix);
+        const double k4 = ks * ks * ks * ks;
+        k_clover_leaves<<<dim3(grid_for(g.V, 128), 6), 128, 0, s>>>(g, FixLinks{UQ, g.lvb}, Gauge64{(double2 *)U64, g.lvb},
+                                                                    k4 * 0x1p59, (double *)Ci64, no_fix);
+        k_clover_assemble<<<grid_for(g.V, 128), 128, 0, s>>>(g, kappa * csw * 0x1p-62 / k4, C64, Ci64, d_bad, no_fix);
         count(2, (double)g.V * (576.0 + 2 * 432.0 + 2 * 576.0));
     }
     k_clover_build<<<grid_for(g.V, 128), 128, 0, s>>>(g, Gauge64{(double2 *)U64, g.lvb}, kappa, csw, C64, Ci64, d_bad,

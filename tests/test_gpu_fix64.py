@@ -264,6 +264,21 @@ def test_clover_build(name, kappa, csw, bent):
     assert (err < 6.7e-15 * cond * (cond if csw > 4 else 1.0)).all()
 
 
+@pytest.mark.parametrize("eps", [0.4, 0.2, 0.1, 0.05, 1e-2, 1e-4, 1e-6])
+def test_clover_build_weak_fields(eps):
+    """The field strength of exp(i eps H): every off-diagonal entry of C, relative to its size over the
+    lattice.  An entry adds up to three planes' Q - Q^+, each four leaves of products whose FP64 sums,
+    here or the oracle's, are good to about 2e-16: 8e-16 for the two."""
+    name = "mid_8^4"
+    dims, block, _, kappa, csw, _, _ = fields(name)
+    U = synth.gauge_field(dims, eps, 43)
+    C = _op(name, U).export_clover().cpu().numpy()
+    ref = O.clover(dims, kappa, csw, U).reshape(C.shape)
+    off = (np.abs(ref).max(axis=0) > 0) & ~np.eye(12, dtype=bool)
+    assert off.sum() == 60
+    assert _worst_component(C[:, off], ref[:, off]) < 8e-16
+
+
 @pytest.mark.parametrize("p", [-455, -400, 400, 470])
 def test_force_scales(p):
     """dS/dU of 2^p phi is 2^(2p) times that of phi: the solves commute with powers of two, and the

@@ -251,14 +251,26 @@ __global__ void __launch_bounds__(128) k_force_plaq(Geom g, Gauge64 U, const dou
 
 // ---- the same products in block fixed point (fix64.cuh), for operators with
 // fixed-point links.  Both kernels form R = X M + S Y, X and Y matrices of FP64
-// numbers brought to one unit (their larger exponent), M and S products of the
-// scaled links: E' = k' E from N and the links, R' = k'^3 R from E' and the pair
-// products.  Matrices whose numbers are not finite or outside the exponents' range
-// take FP64 instructions (force_two_fp64).  24^3 x 48: E 1.04 ms (2.81 with FP64
-// products, at the FP64 pipe's rate), R 2.82 ms (8.52).  Error of R on Gaussian
-// matrices and SU(3) links against exact sums: 6.3e-17 (FP64 sums 1.0e-16).
+// numbers brought to one unit (59 bits below their larger exponent), M and S products
+// of the scaled links: E' = k' E from N and the links, R' = k'^3 R from E' and the
+// pair products.  The products of the low limbs are added too, by their high halves:
+// without them the error was about 9 units of y below, and no line was left between
+// Gaussian matrices and those that need FP64 instructions.
+//
+// Error (emulated against exact sums, Gaussian X and Y, links of eps = 0.4): 0.42
+// units of y in the mean square for E and 0.47 for R, whatever an entry's size; with
+// FP64 instructions 2^-55.1 of the magnitudes, re and im together, of the terms that
+// enter the entry.  The two are equal for terms of 2^54 units.  Matrices with an entry
+// below that (FORCE_LEAST), and ones whose numbers are not finite or outside the
+// exponents' range, run on FP64 instructions, from the links themselves.  Gaussian
+// matrices and their E reach down to 2^55.7 (smallest entry of 2e5 matrices, k' = 1/2,
+// the worst; median 2^58.5).
+// 24^3 x 48: 1.50 ms for E (2.81 with FP64 products, at the FP64 pipe's rate), 3.83
+// for R (8.52); 1.05 and 2.80 without the low limbs' products and the test.  R takes
+// 250 registers, two blocks per SM: three spill 200 B per thread and take 4.16 ms.
+constexpr float FORCE_LEAST = 0x1p49f;  // in units of 2^5 of y
 
-// the limbs of a matrix in units of 2^(K - 1086), |entries| < 2^(K - 1028)
+// the limbs of a matrix in units of 2^(K - 1086), |entries| < 2^(K - 1027)
 __device__ __forceinline__ void f_limbs(const cd *v, int K, FixM3 &o)
 {
 #pragma unroll
@@ -280,60 +292,109 @@ __device__ __forceinline__ int f_exponent(const cd *a, const cd *b)
     return __float_as_int(m) >> 20;
 }
 
-// X M + S Y with FP64 instructions, M and S from their limbs (exact to 2^-60)
-__device__ __noinline__ void force_two_fp64(const cd *X, const int4 *M, const int4 *S, int stride, const cd *Y, cd *R)
+// fix_cmac, and the products of the low limbs as high halves in units of 2^3 of the
+// middle sums: twelve of at most 2^27 keep below 2^31
+__device__ __forceinline__ void f_cmac(int4 u, int4 x, fix_t &hr, fix_t &mr, int &lr, fix_t &hi, fix_t &mi, int &li)
 {
-    auto value = [](int4 v) {
-        return cd{((double)v.x * 0x1p32 + (double)v.y) * 0x1p-60, ((double)v.z * 0x1p32 + (double)v.w) * 0x1p-60};
-    };
-    cd m[9], s[9];
-    for (int k = 0; k < 9; ++k) {
-        m[k] = value(M[k * stride]);
-        s[k] = value(S[k * stride]);
-    }
-    f_m3mul(X, m, R);
-    f_m3mul_acc(s, Y, R);
+    fix_cmac(u, x, hr, mr, hi, mi);
+    const int ur = u.y >> 3, ui = u.w >> 3;
+    lr += __mulhi(ur, x.y);
+    lr += __mulhi(fix_neg(ui), x.w);
+    li += __mulhi(ur, x.w);
+    li += __mulhi(ui, x.y);
 }
 
-// R = X M + S Y, the limbs of M and S at [k stride]; bound: twelve products of a
-// 58-bit and a 60-bit number, middle sums below 12 (2^59 + 2^57) < 2^63
-__device__ __forceinline__ void force_two(const cd *X, const int4 *M, const int4 *S, int stride, const cd *Y, cd *R)
+__device__ __forceinline__ float f_size(int4 v) { return (float)(abs(v.x) + abs(v.z)); }
+
+// The part of R = X M + S Y in fixed point, the limbs of M and S at [k stride];
+// false, and R undefined, when it needs FP64 instructions.  Bounds: the middle sums'
+// a1 b0 twelve times 2^58, their a0 b1 twice sqrt(6) 2^59 (unitary rows), together
+// 2^62.5; y = 2^5 hh at most 2^62.3.
+__device__ __forceinline__ bool force_two(const cd *X, const int4 *M, const int4 *S, int stride, const cd *Y, cd *R)
 {
     const int e = f_exponent(X, Y);
-    if (e >= FIX_EMAX || (e < FIX_EMIN && e > 0)) {
-        cd x[9], y[9], r[9];
-#pragma unroll
-        for (int k = 0; k < 9; ++k) {
-            x[k] = X[k];
-            y[k] = Y[k];
-        }
-        force_two_fp64(x, M, S, stride, y, r);
-#pragma unroll
-        for (int k = 0; k < 9; ++k) R[k] = r[k];
-        return;
-    }
+    if (e >= FIX_EMAX || (e < FIX_EMIN && e > 0)) return false;
     constexpr int L = 5;
-    const int K = max(e, FIX_EMIN) + 6;
+    const int K = max(e, FIX_EMIN) + 5;
     FixM3 fx, fy;
     f_limbs(X, K, fx);
     f_limbs(Y, K, fy);
+    float sx[9], sy[9], t[9];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        sx[k] = f_size(fx.e[k]);
+        sy[k] = f_size(fy.e[k]);
+        t[k] = 0.f;
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            const float m = f_size(M[(k * 3 + j) * stride]), s = f_size(S[(j * 3 + k) * stride]);
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                t[a * 3 + j] = fmaf(m, sx[a * 3 + k], t[a * 3 + j]);
+                t[j * 3 + a] = fmaf(s, sy[k * 3 + a], t[j * 3 + a]);
+            }
+        }
+    float least = t[0];
+#pragma unroll
+    for (int k = 1; k < 9; ++k) least = fminf(least, t[k]);
+    if (least < FORCE_LEAST) return false;
     const double sc = fix_pow2(K - 59 - L);  // hh's unit is 2^(K - 1082)
 #pragma unroll
     for (int a = 0; a < 3; ++a)
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
             fix_t hr = 0, hi = 0, mr = 0x80000000LL >> L, mi = mr;
+            int lr = 0, li = 0;
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
-                fix_cmac(M[(k * 3 + j) * stride], fx.e[a * 3 + k], hr, mr, hi, mi);
-                fix_cmac(S[(a * 3 + k) * stride], fy.e[k * 3 + j], hr, mr, hi, mi);
+                f_cmac(M[(k * 3 + j) * stride], fx.e[a * 3 + k], hr, mr, lr, hi, mi, li);
+                f_cmac(S[(a * 3 + k) * stride], fy.e[k * 3 + j], hr, mr, lr, hi, mi, li);
             }
+            mr = mac64(lr, 8, mr);
+            mi = mac64(li, 8, mi);
             R[a * 3 + j] = cd{sc * __ll2double_rn(fix_join_bits(hr, mr, L)), sc * __ll2double_rn(fix_join_bits(hi, mi, L))};
         }
+    return true;
+}
+
+// the same with FP64 instructions: links n (site, direction, dagger) in loop order;
+// one link: R = scale (X U0 + U0 Y); three: R = scale (X U1 U2 + U0 U1 Y)
+struct ForceLink {
+    int site, dir;
+    bool dag;
+};
+__device__ __noinline__ void force_two_fp64(Gauge64 U, ForceLink l0, ForceLink l1, ForceLink l2, bool three, double scale,
+                                            const cd *X, const cd *Y, cd *R)
+{
+    auto load = [&](ForceLink l, cd *o) {
+        cd u[9];
+        U.load(l.site, l.dir, u);
+        for (int i = 0; i < 3; ++i)
+            for (int j = 0; j < 3; ++j) o[i * 3 + j] = l.dag ? conj(u[j * 3 + i]) : u[i * 3 + j];
+    };
+    cd a[9], b[9], m[9], r[9];
+    load(l0, a);
+    if (three) {
+        load(l1, b);
+        load(l2, m);
+        cd t[9];
+        f_m3mul(b, m, t);
+        f_m3mul(X, t, r);
+        f_m3mul(a, b, t);
+        f_m3mul_acc(t, Y, r);
+    } else {
+        f_m3mul(X, a, r);
+        f_m3mul_acc(a, Y, r);
+    }
+    for (int k = 0; k < 9; ++k) R[k] = scale * r[k];
 }
 
 // k_force_E in fixed point: k' E_mu(x) and k' E_nu(x) of plane p
-__global__ void __launch_bounds__(128, 3) k_force_E_fix(Geom g, FixLinks U, const double2 *N, double2 *Eb)
+__global__ void __launch_bounds__(128, 3) k_force_E_fix(Geom g, FixLinks U, Gauge64 Ud, double ks, const double2 *N,
+                                                        double2 *Eb)
 {
     __shared__ int4 link[9 * 128];
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -354,7 +415,18 @@ __global__ void __launch_bounds__(128, 3) k_force_E_fix(Geom g, FixLinks U, cons
         cd X[9], Y[9], E[9];
         f_N(N, g, c, mu, 0, nu, 0, p, X);
         f_N(N, g, c, mu, s0, nu, s1, p, Y);
-        force_two(X, slot, slot, 128, Y, E);
+        if (!force_two(X, slot, slot, 128, Y, E)) {
+            const ForceLink l = {i, k == 0 ? mu : nu, false};
+            cd x[9], y[9], r[9];
+#pragma unroll
+            for (int e = 0; e < 9; ++e) {
+                x[e] = X[e];
+                y[e] = Y[e];
+            }
+            force_two_fp64(Ud, l, l, l, false, ks, x, y, r);
+#pragma unroll
+            for (int e = 0; e < 9; ++e) E[e] = r[e];
+        }
         double2 *o = Eb + (size_t)(p * 2 + k) * 9 * V + i;
 #pragma unroll
         for (int e = 0; e < 9; ++e) o[e * V] = make_double2(E[e].r, E[e].i);
@@ -363,9 +435,10 @@ __global__ void __launch_bounds__(128, 3) k_force_E_fix(Geom g, FixLinks U, cons
 
 // k_force_plaq in fixed point: k'^3 R_A..R_D from k' E.  With the links in loop
 // order as 0..3 and P_n the product of links n and n + 1, R_n = E_{n+1} P_{n+2} +
-// P_{n+1} E_{n+3}.  The four P stay in shared memory (72 KB, three blocks per SM),
+// P_{n+1} E_{n+3}.  The four P stay in shared memory (72 KB),
 // each thread its own.
-__global__ void __launch_bounds__(128, 3) k_force_plaq_fix(Geom g, FixLinks U, const double2 *Eb, double2 *Rb)
+__global__ void __launch_bounds__(128, 2) k_force_plaq_fix(Geom g, FixLinks U, Gauge64 Ud, double ks, const double2 *Eb,
+                                                           double2 *Rb)
 {
     extern __shared__ int4 prod[];  // [4][9][128]
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -397,8 +470,11 @@ __global__ void __launch_bounds__(128, 3) k_force_plaq_fix(Geom g, FixLinks U, c
 #pragma unroll
             for (int j = 0; j < 3; ++j) {
                 fix_t hr = 0, hi = 0, mr = half, mi = half;
+                int lr = 0, li = 0;
 #pragma unroll
-                for (int m = 0; m < 3; ++m) fix_cmac(A.e[m * 3 + j], P.e[a * 3 + m], hr, mr, hi, mi);
+                for (int m = 0; m < 3; ++m) f_cmac(A.e[m * 3 + j], P.e[a * 3 + m], hr, mr, lr, hi, mi, li);
+                mr = mac64(lr, 8, mr);
+                mi = mac64(li, 8, mi);
                 int4 o;
                 fix_limbs(fix_join_bits(hr, mr, 4), o.x, o.y);
                 fix_limbs(fix_join_bits(hi, mi, 4), o.z, o.w);
@@ -424,7 +500,21 @@ __global__ void __launch_bounds__(128, 3) k_force_plaq_fix(Geom g, FixLinks U, c
         cd X[9], Y[9], R[9];
         getE((k + 1) & 3, X);
         getE((k + 3) & 3, Y);
-        force_two(X, slot + ((k + 2) & 3) * 9 * 128, slot + ((k + 1) & 3) * 9 * 128, 128, Y, R);
+        if (!force_two(X, slot + ((k + 2) & 3) * 9 * 128, slot + ((k + 1) & 3) * 9 * 128, 128, Y, R)) {
+            auto link = [&](int n) {
+                n &= 3;
+                return ForceLink{site(n), n & 1 ? nu : mu, n >= 2};
+            };
+            cd x[9], y[9], r[9];
+#pragma unroll
+            for (int e = 0; e < 9; ++e) {
+                x[e] = X[e];
+                y[e] = Y[e];
+            }
+            force_two_fp64(Ud, link(k + 1), link(k + 2), link(k + 3), true, ks * ks, x, y, r);
+#pragma unroll
+            for (int e = 0; e < 9; ++e) R[e] = r[e];
+        }
         double2 *o = Rb + (size_t)(p * 4 + k) * 9 * V + i;
 #pragma unroll
         for (int e = 0; e < 9; ++e) o[e * V] = make_double2(R[e].r, R[e].i);
@@ -692,10 +782,11 @@ int force(mgc_clover_s *op, const double *phi, double *dSdU, const mgc_solve_par
     const dim3 planes(grid_for(g.V, 128), 6);
     double kc = op->kappa * op->csw / 4.0;
     const FixLinks UQ{op->UQ, g.lvb};
+    const Gauge64 U64{op->gauge->U64, g.lvb};
+    const double ks = std::ldexp(op->kappa, -op->fix_ek);  // the fixed-point links' factor
     if (op->CQ) {
-        const double ks = std::ldexp(op->kappa, -op->fix_ek);
         kc /= ks * ks * ks;
-        k_force_E_fix<<<planes, 128, 0, s>>>(g, UQ, N, Eb);
+        k_force_E_fix<<<planes, 128, 0, s>>>(g, UQ, U64, ks, N, Eb);
     } else {
         k_force_E<<<planes, 128, 0, s>>>(g, Gauge64{op->gauge->U64, g.lvb}, N, Eb);
     }
@@ -704,7 +795,7 @@ int force(mgc_clover_s *op, const double *phi, double *dSdU, const mgc_solve_par
     if (op->CQ) {
         constexpr int smem = 4 * 9 * 128 * sizeof(int4);
         FCUDA(cudaFuncSetAttribute(k_force_plaq_fix, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-        k_force_plaq_fix<<<planes, 128, smem, s>>>(g, UQ, Eb, Rb);
+        k_force_plaq_fix<<<planes, 128, smem, s>>>(g, UQ, U64, ks, Eb, Rb);
     } else {
         k_force_plaq<<<planes, 128, 0, s>>>(g, Gauge64{op->gauge->U64, g.lvb}, Eb, Rb);
     }

@@ -295,6 +295,29 @@ def test_force_scales(p):
     assert rel(_scaled(g1.cpu().numpy(), -2 * p), g0.cpu().numpy()) < 1e-13
 
 
+def test_force_graded_components():
+    """Diagonal links leave the colours apart: with one colour of phi scaled by 2^-p its row and column
+    of the force scale by 2^-p and 4^-p, to the solves' 1e-13 (1e-11 leaves a factor for the condition)."""
+    from paper_2112_00501_gb300 import api
+
+    name = "c4_8^4"
+    dims, block, _, _, csw, _, phi = fields(name)
+    th = np.random.default_rng(9).uniform(-0.6, 0.6, (phi.shape[0], 4, 3))
+    th -= th.mean(axis=2, keepdims=True)
+    U = np.zeros((phi.shape[0], 4, 3, 3), complex)
+    U[..., range(3), range(3)] = np.exp(1j * th)
+    lat = api.Lattice(dims, block, -1)
+    op = api.CloverOperator(api.Gauge(lat, torch.from_numpy(U).cuda(), storage_prec=64), 0.12, csw)
+    par = dict(method=0, smoother_prec=64, tol=1e-13, max_iter=2000)
+    g0 = op.force(torch.from_numpy(phi).cuda(), **par)[0].cpu().numpy()
+    for p in (1, 2, 3, 5, 8, 12, 20, 30, 60):
+        g = op.force(torch.from_numpy(_graded(phi, "colour", p)).cuda(), **par)[0].cpu().numpy()
+        g[..., 2, :] *= 2.0**p
+        g[..., :, 2] *= 2.0**p
+        err = np.linalg.norm(g - g0, axis=(0, 1)) / np.linalg.norm(g0, axis=(0, 1))
+        assert err.max() < 1e-11, (p, err)
+
+
 def test_force_links_without_fixed_point_copy():
     """Bent links: the force's FP64 products, against the oracle's."""
     from paper_2112_00501_gb300 import api

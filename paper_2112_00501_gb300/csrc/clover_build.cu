@@ -7,8 +7,9 @@
 //   C = 1 + i kappa c_SW sum_{mu<nu} sigma_{mu nu} F_{mu nu}.
 // In the chiral basis sigma_{mu nu} = diag(s+_{mu nu}, s-_{mu nu}) with 2x2
 // blocks built from Pauli matrices (table below), so C = diag(C+, C-) with
-// two 6x6 Hermitian blocks; each block is inverted by Gauss-Jordan
-// elimination with partial pivoting.
+// two 6x6 Hermitian blocks.  Each block is inverted by L D L^+ where it is positive
+// definite and the links have a fixed-point copy, by Gauss-Jordan elimination with
+// partial pivoting otherwise.
 #include "fix64.cuh"
 #include "mgc_host.h"
 #include "sigma.cuh"
@@ -505,14 +506,16 @@ __global__ void __launch_bounds__(128, 3) k_clover_assemble(Geom g, double f, do
 #pragma unroll
             for (int b = 0; b < a; ++b, k += 2) A[a * (a + 1) / 2 + b] = cd{pk[k], pk[k + 1]};
         if (invert_hpd6(A)) {
-            // X <- 1 - B X with B = C - 1: where B's rows are shorter than one this
-            // shrinks X's error by their length
+            // X <- 1 - B X with B = C - 1, which multiplies X's error by B: taken where
+            // B's Frobenius norm, and with it its largest eigenvalue, is below one.
+            // Emulated, elimination with pivoting 1.4e-16 to 1.7e-16: 5.5e-17 at a
+            // squared norm of 0.07 (c_SW = 1), 1.0e-16 at 0.95; without the step
+            // 1.2e-16 to 1.4e-16.
             cd X[21];
-            bool shorter = true;
+            double n = 0;
 #pragma unroll
             for (int a = 0; a < 6; ++a) {
                 cd B[6];
-                double n = 0;
 #pragma unroll
                 for (int j = 0; j < 6; ++j) {
                     const int hi = a > j ? a : j, lo = a > j ? j : a, o = 6 + hi * (hi - 1) + 2 * lo;
@@ -520,7 +523,6 @@ __global__ void __launch_bounds__(128, 3) k_clover_assemble(Geom g, double f, do
                     else B[j] = cd{pk[o], a > j ? pk[o + 1] : -pk[o + 1]};
                     n += norm2(B[j]);
                 }
-                shorter = shorter && n < 0.5;
 #pragma unroll
                 for (int b = 0; b <= a; ++b) {
                     cd t = {0, 0};
@@ -532,7 +534,7 @@ __global__ void __launch_bounds__(128, 3) k_clover_assemble(Geom g, double f, do
                     X[a * (a + 1) / 2 + b] = a == b ? cd{1.0 - t.r, 0.0} : -t;
                 }
             }
-            if (shorter)
+            if (n < 1.0)
 #pragma unroll
                 for (int m = 0; m < 21; ++m) A[m] = X[m];
 #pragma unroll

@@ -18,10 +18,10 @@ pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
 
-def _op(name, U=None, kappa=None, tbc=-1):
+def _op(name, U=None, kappa=None, tbc=-1, csw=1.0):
     from paper_2112_00501_gb300 import api
 
-    dims, block, eps, kap, csw, U0, psi = fields(name)
+    dims, block, eps, kap, _, U0, psi = fields(name)
     lat = api.Lattice(dims, block, tbc)
     g = api.Gauge(lat, torch.from_numpy(U0 if U is None else U).cuda(), storage_prec=64)
     return api.CloverOperator(g, kap if kappa is None else kappa, csw)
@@ -277,6 +277,25 @@ def test_clover_build_weak_fields(eps):
     off = (np.abs(ref).max(axis=0) > 0) & ~np.eye(12, dtype=bool)
     assert off.sum() == 60
     assert _worst_component(C[:, off], ref[:, off]) < 8e-16
+
+
+@pytest.mark.parametrize("csw", [1.0, 3.0, 4.5])
+def test_clover_inverse_of_definite_blocks(csw):
+    """C^-1 against extended precision, over the positive definite blocks, no further off than an
+    elimination with pivoting; at the larger c_SW with blocks whose C - 1 has eigenvalues beyond 1
+    among them, where a refining step with C - 1 would not help."""
+    C, Ci = (_op("mid_8^4", csw=csw).export_clover(inverse=i).cpu().numpy() for i in (False, True))
+    blocks = np.concatenate([C[:, :6, :6], C[:, 6:, 6:]])
+    inv = np.concatenate([Ci[:, :6, :6], Ci[:, 6:, 6:]])
+    ev = np.linalg.eigvalsh(blocks)
+    ok = ev[:, 0] > 0.1
+    assert ok.any() and (csw < 4 or (ev[ok, -1] > 2).any())
+    blocks, inv = blocks[ok], inv[ok]
+    lu = np.linalg.inv(blocks)
+    ref, B = lu.astype(np.clongdouble), blocks.astype(np.clongdouble)
+    for _ in range(2):
+        ref = ref + np.einsum("nij,njk->nik", ref, np.eye(6) - np.einsum("nij,njk->nik", B, ref))
+    assert np.linalg.norm(abs(inv - ref).ravel()) < np.linalg.norm(abs(lu - ref).ravel())
 
 
 @pytest.mark.parametrize("p", [-455, -400, 400, 470])

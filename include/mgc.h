@@ -135,11 +135,13 @@ int mgc_gauge_destroy(mgc_gauge_t g);
  * computed on the GPU in FP64 from the gauge field's clover leaves (Sec. 2:
  * computing C and C^-1 from the gauge field); copies of C at FP32 and FP16
  * follow the gauge field's copies.  Where every link is unitary to 1e-3, kappa
- * lies in 2^-16 .. 2^16 and device memory allows, the handle also keeps the
- * links (times kappa) and C as 62-bit fixed-point numbers (1160 bytes a site),
- * on which the FP64 operator, the FP64 smoother's MR and the force run (at
- * least FP64's precision); without them they run on FP64 instructions.  The
- * gauge handle must outlive the operator.  Synchronises stream.
+ * lies in 2^-16 .. 2^16 and 20 times their size stays free on the device, the
+ * handle also keeps the links (times kappa) and C as 62-bit fixed-point numbers
+ * (1160 bytes a site), on which the FP64 operator, the FP64 smoother's MR and the
+ * force run; without them they run on FP64 instructions, and with them wherever a
+ * component of the result is too small beside its neighbourhood for fixed point to
+ * be as precise as those (such fields take up to 1.5 times as long as without the
+ * copies).  The gauge handle must outlive the operator.  Synchronises stream.
  */
 int mgc_clover_create(mgc_gauge_t g, double kappa, double csw, void *stream, mgc_clover_t *out);
 int mgc_clover_destroy(mgc_clover_t op);

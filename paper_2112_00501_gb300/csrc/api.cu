@@ -298,11 +298,29 @@ int mgc_clover_create(mgc_gauge_t g, double kappa, double csw, void *stream, mgc
     CCUDA(cudaMalloc(&op->Ci64, clover_bytes(geo, 64)));
     CCUDA(cudaMalloc(&d_bad, 3 * sizeof(int)));
     CCUDA(cudaMemsetAsync(d_bad, 0, 3 * sizeof(int), s));
-    // fixed-point copies for the FP64 operator, for hopping parameters of ordinary
-    // size and where there is room for them (it runs without)
+    // C and C^-1 (the latter for the clover-preconditioned operator A = C^-1 D)
+    // at every precision the gauge field keeps
+    if (g->prec <= 32) {
+        CCUDA(cudaMalloc(&op->C32, clover_bytes(geo, 32)));
+        CCUDA(cudaMalloc(&op->Ci32, clover_bytes(geo, 32)));
+    }
+    if (g->prec == 16) {
+        CCUDA(cudaMalloc(&op->C16, clover_bytes(geo, 16)));
+        op->C16_sc = (float *)((uint4 *)op->C16 + (size_t)geo.V * 9);
+        CCUDA(cudaMalloc(&op->Ci16, clover_bytes(geo, 16)));
+        op->Ci16_sc = (float *)((uint4 *)op->Ci16 + (size_t)geo.V * 9);
+    }
+    // Fixed-point copies for the FP64 operator, for hopping parameters of ordinary
+    // size and where they leave 20 times their size free (23 kB a site, what a force
+    // evaluation whose solves keep 32 FP64 directions allocates): they cannot be
+    // given up later, when a captured graph may hold their addresses, so a call that
+    // fits without them must not run out of memory for them.
     const double ks = std::frexp(kappa, &op->fix_ek);
     if (fabs(kappa) >= 0x1p-16 && fabs(kappa) <= 0x1p16) {
-        if (cudaMalloc(&op->UQ, gauge_bytes(geo, 64, 18)) != cudaSuccess ||
+        const size_t bytes = gauge_bytes(geo, 64, 18) + clover_bytes(geo, 64) + (size_t)geo.V * sizeof(int2);
+        size_t avail = 0, total = 0;
+        if (cudaMemGetInfo(&avail, &total) != cudaSuccess || avail / 21 < bytes ||
+            cudaMalloc(&op->UQ, gauge_bytes(geo, 64, 18)) != cudaSuccess ||
             cudaMalloc(&op->CQ, clover_bytes(geo, 64)) != cudaSuccess ||
             cudaMalloc(&op->CE, (size_t)geo.V * sizeof(int2)) != cudaSuccess) {
             (void)cudaGetLastError();
@@ -317,23 +335,15 @@ int mgc_clover_create(mgc_gauge_t g, double kappa, double csw, void *stream, mgc
     if (st) return bail(st);
     if (op->CQ) st = launch_fix_clover(geo, op->C64, op->fix_ek, op->CQ, op->CE, d_bad + 1, s);
     if (st) return bail(st);
-    // C and C^-1 (the latter for the clover-preconditioned operator A = C^-1 D)
-    // at every precision the gauge field keeps
     if (g->prec <= 32) {
-        CCUDA(cudaMalloc(&op->C32, clover_bytes(geo, 32)));
         st = launch_clover_lowprec(geo, op->C64, 32, op->C32, s);
         if (st) return bail(st);
-        CCUDA(cudaMalloc(&op->Ci32, clover_bytes(geo, 32)));
         st = launch_clover_lowprec(geo, op->Ci64, 32, op->Ci32, s);
         if (st) return bail(st);
     }
     if (g->prec == 16) {
-        CCUDA(cudaMalloc(&op->C16, clover_bytes(geo, 16)));
-        op->C16_sc = (float *)((uint4 *)op->C16 + (size_t)geo.V * 9);
         st = launch_clover_lowprec(geo, op->C64, 16, op->C16, s);
         if (st) return bail(st);
-        CCUDA(cudaMalloc(&op->Ci16, clover_bytes(geo, 16)));
-        op->Ci16_sc = (float *)((uint4 *)op->Ci16 + (size_t)geo.V * 9);
         st = launch_clover_lowprec(geo, op->Ci64, 16, op->Ci16, s);
         if (st) return bail(st);
     }

@@ -151,6 +151,32 @@ def test_graded_components(eps, axis):
         assert _worst_component(op.A(x, 64).cpu().numpy(), ref) < 1e-15, p
 
 
+def test_copies_leave_room_for_workspaces():
+    """With 2 GB free an operator on 16^3 x 32 makes no copies (152 MB, which want 20 times as much
+    left) and gives the same results."""
+    from paper_2112_00501_gb300 import api
+
+    dims, block, _, kappa, csw, U, psi = fields("c1_16^3x32")
+    g = api.Gauge(api.Lattice(dims, block, -1), torch.from_numpy(U).cuda(), storage_prec=64)
+    x = torch.from_numpy(psi).cuda()
+
+    def create():
+        before = torch.cuda.mem_get_info()[0]
+        op = api.CloverOperator(g, kappa, csw)
+        return before - torch.cuda.mem_get_info()[0], op.D(x, prec=64).cpu().numpy()
+
+    create()  # the kernels' local memory
+    torch.cuda.empty_cache()
+    roomy, y = create()
+    torch.cuda.empty_cache()
+    hold = torch.empty(torch.cuda.mem_get_info()[0] - (2 << 30), dtype=torch.uint8, device="cuda")
+    tight, z = create()
+    del hold
+    torch.cuda.empty_cache()
+    assert roomy - tight > 0.9 * 1160 * psi.shape[0]
+    assert rel(z, y) < 6e-16
+
+
 def test_batch_is_bit_identical():
     """A batch of one lattice with a fixed-point copy and one without."""
     from paper_2112_00501_gb300 import api

@@ -457,7 +457,10 @@ int mgc_batch_tune(mgc_batch_t b, int prec, int force, int *rhs_per_thread, int 
                    int *rhs_fast_sap, void *stream);
 /*
  * Pin the launch shape at precision prec instead of tuning: rhs_per_thread
- * 1, 2 or 4; threads 128 or 256; rhs_fast_d, rhs_fast_sap 0 or 1.
+ * 1, 2 or 4; threads 128 or 256; rhs_fast_d, rhs_fast_sap 0 or 1.  At precision
+ * 64 a batch with an operator that has fixed-point copies (mgc_clover_create)
+ * runs with one right-hand side per thread and 128 threads whatever is pinned;
+ * tuning it gives those.
  */
 int mgc_batch_set_shape(mgc_batch_t b, int prec, int rhs_per_thread, int threads, int rhs_fast_d,
                         int rhs_fast_sap);

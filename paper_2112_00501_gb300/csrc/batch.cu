@@ -507,10 +507,14 @@ int run_tune(mgc_batch_s *B, int prec)
     };
     float best = 1e30f;
     const int rbs[3] = {1, 2, 4};
-    for (int a = 0; a < 3 && st == MGC_OK; ++a) {
+    // with an operator's fixed-point copies in it the FP64 launch has one shape, 1 and
+    // 128, and only the order of its blocks varies
+    bool shaped = true;
+    for (int k = 0; k < n; ++k) shaped = shaped && (prec != 64 || !B->spec.ops[k]->CQ);
+    for (int a = 0; a < (shaped ? 3 : 1) && st == MGC_OK; ++a) {
         const int rb = rbs[a];
         if (rb > 1 && (rb + 1) / 2 >= maxr) continue;  // 2 needs >= 2 rhs, 4 needs >= 3
-        for (int threads = 128; threads <= 256 && st == MGC_OK; threads *= 2)
+        for (int threads = 128; threads <= (shaped ? 256 : 128) && st == MGC_OK; threads *= 2)
             for (int rf = 0; rf <= 1 && st == MGC_OK; ++rf) {
                 if (rf == 1 && maxr <= rb) continue;  // one group per site block: the order is the same
                 const BatchSpec sp = spec_with(B, rf);

@@ -199,6 +199,25 @@ def test_batch_is_bit_identical():
                 assert torch.equal(o, (op.apply_Ddag if dagger else op.apply_D)(p, 64, n))
 
 
+def test_batch_shape_with_copies():
+    """A launch with copies has one shape, whatever is pinned; a batch without is tuned over all."""
+    from paper_2112_00501_gb300 import api
+
+    name = "mid_8^4"
+    bent = fields(name)[5].copy()
+    bent[5, 2] *= 1.01
+    op, plain = _op(name), _op(name, bent)
+    x = op.lattice.pack(torch.from_numpy(np.stack([fields(name)[6]] * 3)).cuda(), 64)
+    for ops in ([op, op], [op, plain], [plain, plain]):
+        batch = api.Batch(ops, [3, 3])
+        t = batch.tune(64)
+        assert plain is ops[0] or (t["rhs_per_thread"], t["threads"]) == (1, 128)
+        ref = [o.apply_D(x, 64, 3) for o in ops]
+        for shape in ((1, 128), (2, 256), (4, 128)):
+            batch.set_shape(64, *shape, 1, 0)
+            assert all(torch.equal(a, b) for a, b in zip(batch.apply_D([x, x], 64), ref))
+
+
 def _check_sap(name, b, kappa=None, n_cy=2, n_mr=4, x0=None, p=0, tol=2e-15):
     dims, block, eps, kap, csw, U, _ = fields(name)
     kappa = kap if kappa is None else kappa

@@ -238,10 +238,11 @@ __device__ __forceinline__ void leaf_terms(const FixM3 &P, const FixM3 &A, float
         }
 }
 
-// The same nine reals with FP64 instructions from the links themselves, scale =
-// 2^59 k'^4
-__device__ __noinline__ void leaves_fp64(Geom g, Gauge64 U, int x, int mu, int nu, double scale, double *G)
+// The same nine reals with FP64 instructions from the links themselves, in units of
+// 2^-59
+__device__ __noinline__ void leaves_fp64(Geom g, Gauge64 U, int x, int mu, int nu, double *G)
 {
+    const double scale = 0x1p59;
     int c[4];
     site_coords(g, x, c);
     cd Q[9];
@@ -255,9 +256,10 @@ __device__ __noinline__ void leaves_fp64(Geom g, Gauge64 U, int x, int mu, int n
         }
 }
 
-// Q - Q^+ of plane blockIdx.y at every site, Q the sum of its four leaves of the
-// scaled links: three imaginary diagonals and the entries (1,0), (2,0), (2,1), nine
-// reals in units of 2^-59, to F as reals 9 plane + k of a packed clover term.
+// Q - Q^+ of plane blockIdx.y at every site, Q the sum of its four leaves, from those
+// of the scaled links times unscale = 1 / k'^4: three imaginary diagonals and the
+// entries (1,0), (2,0), (2,1), nine reals in units of 2^-59, to F as reals 9 plane + k
+// of a packed clover term.
 // Their error is some units whatever their size, with FP64 instructions it goes with
 // the terms' magnitudes: fields exp(i eps H) have the same error, 2.6e-16 of the
 // off-diagonal reals, at eps = 0.11.  A site and plane with a real whose terms (those
@@ -265,7 +267,7 @@ __device__ __noinline__ void leaves_fp64(Geom g, Gauge64 U, int x, int mu, int n
 // fields of eps >= 0.3 do not (smallest of 1.5e5 reals 2^55.4; k' = 1/2, the worst),
 // is computed with FP64 instructions.
 constexpr float LEAF_LEAST = 0x1p52f;  // 2^55 units
-__global__ void __launch_bounds__(128, 4) k_clover_leaves(Geom g, FixLinks U, Gauge64 Ud, double scale, double *F,
+__global__ void __launch_bounds__(128, 4) k_clover_leaves(Geom g, FixLinks U, Gauge64 Ud, double unscale, double *F,
                                                           const int *no_fix)
 {
     __shared__ float terms[9 * 128];
@@ -340,10 +342,10 @@ __global__ void __launch_bounds__(128, 4) k_clover_leaves(Geom g, FixLinks U, Ga
     for (int k = 0; k < 9; ++k) fine = fine && S[k * 128] >= LEAF_LEAST;
     if (fine) {
 #pragma unroll
-        for (int k = 0; k < 9; ++k) put(k, __ll2double_rn(G[k]));
+        for (int k = 0; k < 9; ++k) put(k, unscale * __ll2double_rn(G[k]));
     } else {
         double D[9];
-        leaves_fp64(g, Ud, x, mu, nu, scale, D);
+        leaves_fp64(g, Ud, x, mu, nu, D);
         for (int k = 0; k < 9; ++k) put(k, D[k]);
     }
 }
@@ -423,7 +425,7 @@ __device__ __noinline__ bool invert_general(const double *pk, double *out)
 }
 
 // C = 1 + f sum sigma i (Q - Q^+) and C^-1 from k_clover_leaves' reals, f = kappa
-// c_SW 2^-62 / k'^4; Ci64 holds those reals on entry
+// c_SW 2^-62; Ci64 holds those reals on entry
 __global__ void __launch_bounds__(128, 3) k_clover_assemble(Geom g, double f, double2 *C64, double2 *Ci64, int *bad,
                                                          const int *no_fix)
 {
@@ -566,10 +568,9 @@ int launch_clover_build(const Geom &g, const double2 *U64, const int4 *UQ, doubl
                         double csw, double2 *C64, double2 *Ci64, int *d_bad, cudaStream_t s)
 {
     if (UQ) {
-        const double k4 = ks * ks * ks * ks;
         k_clover_leaves<<<dim3(grid_for(g.V, 128), 6), 128, 0, s>>>(g, FixLinks{UQ, g.lvb}, Gauge64{(double2 *)U64, g.lvb},
-                                                                    k4 * 0x1p59, (double *)Ci64, no_fix);
-        k_clover_assemble<<<grid_for(g.V, 128), 128, 0, s>>>(g, kappa * csw * 0x1p-62 / k4, C64, Ci64, d_bad, no_fix);
+                                                                    1 / (ks * ks * ks * ks), (double *)Ci64, no_fix);
+        k_clover_assemble<<<grid_for(g.V, 128), 128, 0, s>>>(g, kappa * csw * 0x1p-62, C64, Ci64, d_bad, no_fix);
         count(2, (double)g.V * (576.0 + 2 * 432.0 + 2 * 576.0));
     }
     k_clover_build<<<grid_for(g.V, 128), 128, 0, s>>>(g, Gauge64{(double2 *)U64, g.lvb}, kappa, csw, C64, Ci64, d_bad,

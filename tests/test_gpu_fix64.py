@@ -324,6 +324,24 @@ def test_clover_build_weak_fields(eps):
     assert _worst_component(C[:, off], ref[:, off]) < 8e-16
 
 
+@pytest.mark.parametrize("kappa", [0.125, 0.1])
+def test_singular_clover_block_is_refused(kappa):
+    """A plaquette of diag(i, -i, 1) in every (x, y) plane gives C = 1 -+ kappa c_SW diag(1, -1, 0) in
+    FP64 without rounding, singular at kappa c_SW = 1 (0.1 * 10 is 1 after rounding too)."""
+    from paper_2112_00501_gb300 import _lib, api
+
+    dims, block = (8, 4, 4, 4), (4, 2, 2, 2)
+    x = np.arange(512) % 8
+    U = np.broadcast_to(np.eye(3), (512, 4, 3, 3)).astype(complex).copy()
+    U[:, 1, 0, 0] = np.array([1, 1j, -1, -1j])[x % 4]
+    U[:, 1, 1, 1] = U[:, 1, 0, 0].conj()
+    g = api.Gauge(api.Lattice(dims, block, -1), torch.from_numpy(U).cuda(), storage_prec=64)
+    with pytest.raises(_lib.MgcError) as e:
+        api.CloverOperator(g, kappa, round(1 / kappa))
+    assert e.value.status == _lib.MGC_ERR_BREAKDOWN
+    api.CloverOperator(g, kappa, 0.5 / kappa)
+
+
 @pytest.mark.parametrize("csw", [1.0, 3.0, 4.5])
 def test_clover_inverse_of_definite_blocks(csw):
     """C^-1 against extended precision, over the positive definite blocks, no further off than an

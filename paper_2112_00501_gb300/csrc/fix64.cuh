@@ -301,8 +301,15 @@ __device__ __forceinline__ void fix_project_limbs(Q q, int m, bool back, int h1[
 // of: 18 % of its FP64 solve in spills.)
 struct FixTerms {
     int n[3];
-    int hops;
-    __device__ __forceinline__ void clear() { n[0] = n[1] = n[2] = hops = 0; }
+    int hops;  // those added, less NONE while the site itself adds nothing
+    static constexpr int NONE = 16;
+    __device__ __forceinline__ void clear(bool own)
+    {
+        n[0] = n[1] = n[2] = 0;
+        hops = own ? 0 : -NONE;
+    }
+    // nothing has been added: the sum is zero
+    __device__ __forceinline__ bool nothing() const { return hops == -NONE; }
     // the unit grows by 2^d
     __device__ __forceinline__ void shift(int d)
     {
@@ -324,7 +331,7 @@ struct FixTerms {
     // whether every component of the sum acc has `least` counts
     __device__ __forceinline__ bool enough(int least, const Cx<fix_t> acc[12]) const
     {
-        if (all_reach(least)) return true;
+        if (all_reach(least) || nothing()) return true;
         bool all = true;
 #pragma unroll
         for (int k = 0; k < 12; ++k) all = all && reaches(least, k, acc[k]);
@@ -334,7 +341,8 @@ struct FixTerms {
     // hops (whose sum's error is 1.2 units), for fewer by the square root of their number
     __device__ __forceinline__ int least() const
     {
-        return hops > 4 ? 1 << 22 : (hops > 2 ? 0x2d4000 : (hops > 1 ? 1 << 21 : 0x16a000));
+        const int h = hops & (NONE - 1);
+        return h > 4 ? 1 << 22 : (h > 2 ? 0x2d4000 : (h > 1 ? 1 << 21 : 0x16a000));
     }
 };
 
@@ -568,7 +576,7 @@ __device__ __forceinline__ bool fix_dirac_sum(const Geom &g, int i, const Spinor
     fix_commit();
 
     int state = FIX_HOP;
-    terms.clear();
+    terms.clear(false);
     if constexpr (CLOVER) {
         FixRaw r;
         r.load(in, i);
@@ -577,6 +585,7 @@ __device__ __forceinline__ bool fix_dirac_sum(const Geom &g, int i, const Spinor
         const int ep = max(r.emax, FIX_EMIN);
         E = ep + eC.y;
         if (fix_in_range(r, ep)) {
+            terms.clear(true);
             fix_clover(C, i, [&](int k) { return fix_component(r, k, ep + 4); }, eC.x - eC.y, acc);
         } else {
             state = fix_all_zero(r) ? FIX_ZERO : FIX_LEAVE;

@@ -373,8 +373,8 @@ __global__ void __launch_bounds__(256) k_sap_colour(Geom g, SP b, SP x, GA U, CL
 // widening products in turn.  r and e in shared memory (98 KB) and 128 registers
 // give two blocks per SM; the residual's staging slots lie over r and e, which
 // come later.  16^3 x 32, 4 steps from a guess: 373 us a colour (356 us without the
-// tests of the components' sizes) against 910 us with FP64 instructions.  Error of two sweeps against quadruple precision on 8^4: 1.0e-16
-// against 2.3e-16.
+// tests of the components' sizes) against 910 us with FP64 instructions.  Error of two
+// sweeps against quadruple precision on 8^4: 1.0e-16 against 2.3e-16.
 
 // the largest biased exponent of 24 reals
 __device__ __forceinline__ int fix_exponent(const Cx<double> v[12])
@@ -546,7 +546,7 @@ __global__ void __launch_bounds__(256, 2) k_sap_fix(Geom g, Spinor64 b, Spinor64
         FixTerms terms;
         int E;
         bool done = fix_dirac_sum<false>(g, i, xx, U, C, reinterpret_cast<int4 *>(smem) + l, vb, acc, terms, E);
-        if (done && !terms.all_reach(terms.least())) {
+        if (done && !terms.all_reach(terms.least()) && !terms.nothing()) {
             // b is a term of b - D x as well (high words order like the doubles)
             const int b0 = __double2hiint(fix_pow2(E + C.ek - 55 + 32) * terms.least());
 #pragma unroll
@@ -600,7 +600,7 @@ __global__ void __launch_bounds__(256, 2) k_sap_fix(Geom g, Spinor64 b, Spinor64
 #pragma unroll
         for (int k = 0; k < 12; ++k) acc[k] = -acc[k];
         FixTerms terms;
-        terms.clear();
+        terms.clear(true);
 #pragma unroll 1
         for (int d = 0; d < 8; ++d) {
             const int mu = d >> 1;

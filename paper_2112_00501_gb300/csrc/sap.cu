@@ -23,9 +23,10 @@
 // preconditioned MR of DD-alphaAMG: the even sites (the first half of a domain
 // in the packed order) run MR on the Schur complement
 // C_ee - kappa^2 H_eo C_oo^-1 H_oe with source r_e + kappa H_eo C_oo^-1 r_o,
-// the odd sites apply C_oo^-1 (read from global memory) in between and finally
-// form e_o = C_oo^-1 (r_o + kappa H_oe e_e).  Odd entries of the shared vector
-// hold the odd-site intermediate, even entries the even-site residual.
+// the odd sites apply C_oo^-1 (read from global memory at FP64, kept in shared
+// memory by k_sap_eo) in between and finally form
+// e_o = C_oo^-1 (r_o + kappa H_oe e_e).  Odd entries of the shared vector hold the
+// odd-site intermediate, even entries the even-site residual.
 #include "fix64.cuh"
 #include "hop.cuh"
 #include "hop16.cuh"
@@ -365,9 +366,15 @@ __global__ void __launch_bounds__(256) k_sap_colour(Geom g, SP b, SP x, GA U, CL
 // are FP64 as before, on the integers' doubles r' and p': with
 // beta = <p', r'>/<p', p'>, alpha = -beta 2^(-4 - ek) and r - alpha p is
 // 2^(E - 1082) (r' - beta p').  A domain whose residual is not finite or outside
-// 2^-894 .. 2^961, or one where a component of D_B r is too small for the unit at
-// any step (SAP_FIX_LEAST), is solved with FP64 instructions instead
-// (sap_domain_fp64); at a site of the residual the source b counts as a term too.
+// 2^-894 .. 2^961, or one where a component of D_B r is too small for the unit
+// (SAP_FIX_LEAST) at the first step or at one whose r has grown, is solved with
+// FP64 instructions instead (sap_domain_fp64).  The source b counts as a term too, of
+// the residual and, where there is a guess, of D_B r, since r = b - D x has b's rounding
+// error at least; and later steps' errors are no larger than the one that was accepted
+// at the first (with FP64 instructions r carries r_0's rounding along as well).  Without
+// these two, domains whose r is largest at their faces, in their middle or at a site
+// with a nearly singular C (after a sweep at small kappa, of many steps or at large
+// c_SW) went to FP64 instructions.
 //
 // Bound: FP64 pipe (56 % busy; conversions, inner products and updates) and the
 // widening products in turn.  r and e in shared memory (98 KB) and 128 registers
@@ -502,9 +509,28 @@ constexpr size_t sap_fix_smem(int vb) { return (size_t)vb * 24 * 16 + 96 * sizeo
 
 // The counts (FixTerms) that every component of D_B r needs: 2^52 units.  The unit
 // is the whole domain's here and corner sites have four hops, so that Gaussian
-// residuals reach down to 2^53.5 (4e5 components, four steps; median 2^56.8); at
-// 2^53 one domain in 10^4 would leave, each holding its launch up by 300 us.
+// residuals reach down to about 2^53.5 (4e5 components, four steps; median 2^56.8).  At
+// 2^52 none of the 20,480 domain solves of an FP64 solve on 16^3 x 32 leaves; at 2^53
+// one in 10^4 would, by the tail of that distribution, each holding its launch up by
+// the 300 us of a domain solve with FP64 instructions.
 constexpr int SAP_FIX_LEAST = 1 << (52 - 32);
+
+// whether every component of the sum acc, or the source b's, has `least` counts; unit:
+// the biased exponent of acc's unit, 0x7ff to leave b out
+__device__ __forceinline__ bool reach_with_b(const FixTerms &terms, int least, const Cx<fix_t> acc[12], const Spinor64 &b,
+                                             int i, int unit)
+{
+    // high words order like the doubles
+    const int b0 = unit < 0x7ff ? __double2hiint(fix_pow2(unit + 32) * least) : 0x7fffffff;
+    bool all = true;
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+        const double2 v = b.at(i)[(size_t)k << b.lvb];
+        all = all && (terms.reaches(least, k, acc[k]) ||
+                      max(__double2hiint(v.x) & 0x7fffffff, __double2hiint(v.y) & 0x7fffffff) >= b0);
+    }
+    return all;
+}
 
 template <int LVB>
 __global__ void __launch_bounds__(256, 2) k_sap_fix(Geom g, Spinor64 b, Spinor64 x, FixLinks U, FixClover C, Gauge64 Ud,
@@ -546,16 +572,8 @@ __global__ void __launch_bounds__(256, 2) k_sap_fix(Geom g, Spinor64 b, Spinor64
         FixTerms terms;
         int E;
         bool done = fix_dirac_sum<false>(g, i, xx, U, C, reinterpret_cast<int4 *>(smem) + l, vb, acc, terms, E);
-        if (done && !terms.all_reach(terms.least()) && !terms.nothing()) {
-            // b is a term of b - D x as well (high words order like the doubles)
-            const int b0 = __double2hiint(fix_pow2(E + C.ek - 55 + 32) * terms.least());
-#pragma unroll
-            for (int k = 0; k < 12; ++k) {
-                const double2 v = bb.at(i)[(size_t)k << b.lvb];
-                done = done && (terms.reaches(terms.least(), k, acc[k]) ||
-                                max(__double2hiint(v.x) & 0x7fffffff, __double2hiint(v.y) & 0x7fffffff) >= b0);
-            }
-        }
+        if (done && !terms.all_reach(terms.least()) && !terms.nothing())
+            done = reach_with_b(terms, terms.least(), acc, bb, i, E + C.ek - 55);
         if (done) {
             const double sc = fix_pow2(E + C.ek - 55);
             bb.load(i, rv);
@@ -624,7 +642,10 @@ __global__ void __launch_bounds__(256, 2) k_sap_fix(Geom g, Spinor64 b, Spinor64
                 fix_hop(U.at(back ? blkbase | ln : i, mu), vb, d, back, h1, h0, acc, terms);
             }
         }
-        fp64 = !terms.enough(SAP_FIX_LEAST, acc);
+        // with a unit no larger than the first step's, this one's error is no larger than
+        // the one that was accepted there
+        if ((it == 0 || E > e0 + dE) && !terms.all_reach(SAP_FIX_LEAST))
+            fp64 = !reach_with_b(terms, SAP_FIX_LEAST, acc, bb, i, x_zero ? 0x7ff : E + C.ek - 55);
         // inner products of p' and r' (the integers as doubles), then r' - beta p'
         double pr = 0, pi = 0, pp = 0;
         Cx<double> p[12];
@@ -2413,9 +2434,9 @@ static int sap_run(const Geom &g, SP b, SP x, GA U, CL C, CL Ci, double kappa, i
 }
 
 // The largest room the fixed-point MR leaves for the clover term: beyond it (kappa
-// below about 1/250) the hops are so small in the domain's unit that most domains
-// would find a component too small (SAP_FIX_LEAST) and run on FP64 after all.
-constexpr int SAP_FIX_MAX_ROOM = 3;
+// below about 1/1000) r would keep less than FP64's 53 bits below the domain's largest
+// component.
+constexpr int SAP_FIX_MAX_ROOM = 6;
 
 template <int LVB>
 static int sap_run_fix(const mgc_clover_s *op, const void *b, void *x, int nrhs, int n_cy, int n_mr, int x_is_zero,
@@ -2440,7 +2461,7 @@ static int sap_run_fix(const mgc_clover_s *op, const void *b, void *x, int nrhs,
 }
 
 // the smoother: MR on D_B (clover C), Jacobi on A_B (clover C^-1) or even-odd
-// MR on D_B (clover C, odd-site C^-1 from global memory)
+// MR on D_B (clover C, C^-1 at the odd sites)
 template <int MODE>
 static int sap_launch_impl(const mgc_clover_s *op, int prec, const void *b, void *x, int nrhs, int n_cy, int n_it,
                            int x_is_zero, cudaStream_t s)

@@ -273,6 +273,18 @@ def test_sap_step_counts(n_mr):
     _check_sap("ragged_8x4x12x8", fields("ragged_8x4x12x8")[6], n_cy=1, n_mr=n_mr)
 
 
+@pytest.mark.parametrize("kappa,n_mr", [(0.02, 4), (0.05, 4), (0.1355, 12)])
+def test_sap_second_sweep_residuals(kappa, n_mr):
+    """Residuals that the first sweep leaves at the faces of the domains: every component of the second
+    sweep's result to the bound of test_sap_graded_components."""
+    name = "mid_8^4"
+    dims, block, _, _, csw, U, b = fields(name)
+    op = _op(name, kappa=kappa)
+    got = op.sap(torch.from_numpy(b).cuda(), 64, 2, n_mr).cpu().numpy()
+    ref = O.sap(dims, block, -1, kappa, U, op.export_clover().cpu().numpy(), b, ncy=2, nmr=n_mr)
+    assert _worst_component(got, ref) < 1e-14
+
+
 @pytest.mark.parametrize("p", [-880, -400, 400, 955])
 def test_sap_scales(p):
     _check_sap("mid_8^4", fields("mid_8^4")[6], p=p)
@@ -291,8 +303,8 @@ def test_sap_sparse_and_zero_domains():
 
 @pytest.mark.parametrize("eps", [0.0, 1e-5])
 @pytest.mark.parametrize("axis", ["colour", "spin"])
-@pytest.mark.parametrize("n_cy,n_mr", [(1, 1), (2, 4)])
-def test_sap_graded_components(eps, axis, n_cy, n_mr):
+@pytest.mark.parametrize("n_cy,n_mr,guess", [(1, 1, False), (2, 4, False), (1, 4, True)])
+def test_sap_graded_components(eps, axis, n_cy, n_mr, guess):
     """As test_graded_components, for the smoother.  Every component carries alpha's error: the oracle
     adds a domain's N = 3072 products one after another, a random walk of sqrt(N) u = 6e-15 in <p, r>
     and in <p, p>, together 9e-15.  (Without a test of the sizes a colour at 2^-20 was off by 2e-11.)"""
@@ -303,8 +315,10 @@ def test_sap_graded_components(eps, axis, n_cy, n_mr):
     Cl = op.export_clover().cpu().numpy()
     for p in (0, 1, 2, 3, 4, 5, 7, 10, 15, 20, 25, 40, 60):
         b = _graded(psi, axis, p)
-        got = op.sap(torch.from_numpy(b).cuda(), 64, n_cy, n_mr).cpu().numpy()
-        ref = O.sap(dims, block, -1, kappa, U, Cl, b, ncy=n_cy, nmr=n_mr)
+        x0 = np.roll(b, 7, axis=0) if guess else None
+        xg = torch.from_numpy(x0).cuda() if guess else None
+        got = op.sap(torch.from_numpy(b).cuda(), 64, n_cy, n_mr, x0=xg).cpu().numpy()
+        ref = O.sap(dims, block, -1, kappa, U, Cl, b, x0=x0, ncy=n_cy, nmr=n_mr)
         assert _worst_component(got, ref) < 1e-14, p
 
 

@@ -181,9 +181,10 @@ __global__ void k_clover_build(Geom g, Gauge64 U, double kappa, double csw, doub
 // ---- the build from the fixed-point links (fix64.cuh): the leaves' matrix
 // products on the integer multiply-add units, one thread per site and plane, then
 // C and C^-1 per site with FP64 instructions.  24^3 x 48: 2.2 and 2.3 ms (leaves of
-// weak fields, which run on FP64 instructions, 8.8 ms), against 19.1 ms with FP64 products, a generic sigma table and Gauss-Jordan elimination
-// throughout, bound by the FP64 pipe.  Error of C^-1 against quadruple precision:
-// 9.4e-17 (1.5e-16 by elimination).
+// weak fields, which run on FP64 instructions, 8.8 ms), against 19.1 ms with FP64
+// products, a generic sigma table and Gauss-Jordan elimination throughout, bound by
+// the FP64 pipe.  Error of C^-1 against quadruple precision: 9.4e-17 (1.5e-16 by
+// elimination).
 
 // the links of the four leaves at x in the plane (mu, nu) in loop order: the
 // shifts (dm, dn) of the link's site, its direction (0: mu, 1: nu), its dagger

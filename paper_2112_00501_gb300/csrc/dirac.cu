@@ -194,10 +194,10 @@ __device__ __forceinline__ int2 fix_store(fix_t q)
     return make_int2(hi, max(lo, -0x7fffffff));
 }
 
-// The links times ks (0 < |ks| < 1, as ks62 = ks 2^62) in units of 2^-60, rounded to
-// nearest; *bad is set unless every link is unitary to 1e-3 (norms of its rows and
-// columns, products of its rows), which bounds the operator's sums and those of the
-// links' products: with unit norms alone, four-link products could reach three
+// The links (at 2^-62) times ks (0 < |ks| < 1, as ks62 = ks 2^62) in units of 2^-60,
+// rounded to nearest; *bad is set unless every link is unitary to 1e-3 (norms of its
+// rows and columns, products of its rows), which bounds the operator's sums and those
+// of the links' products: with unit norms alone, four-link products could reach three
 // times a unitary field's, beyond the clover leaves' 64 bits.
 __global__ void k_fix_links(Geom g, Gauge64 U, long long ks62, int4 *__restrict__ out, int *bad)
 {
@@ -237,8 +237,8 @@ __global__ void k_fix_links(Geom g, Gauge64 U, long long ks62, int4 *__restrict_
 }
 
 // C in units of 2^(e + ek - 60) with the site's exponent e, |C| < 2^(e + ek) and a
-// row's absolute sum below four times that, and the bits room that the sum's unit leaves for it: a row's absolute sum is below
-// 2^(5 + room + ek).
+// row's absolute sum below four times that, and the bits room that the sum's unit
+// leaves for it: a row's absolute sum is below 2^(5 + room + ek).
 __global__ void k_fix_clover(Geom g, Clover64 C, int ek, int4 *__restrict__ out, int2 *__restrict__ ex, int *bad)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;

@@ -3,8 +3,8 @@
 //
 // GB300 issues 2 FP64 fused multiply-adds per clock and SM, but 32 widening
 // integer multiply-adds (32 x 32 + 64 bits; the first measured with eight
-// independent chains per thread, the second from the busy cycles of the pipe).  A product of two-limb integers
-// a = a1 2^32 + a0 whose low limbs are balanced (|a0| <= 2^31, random sign)
+// independent chains per thread, the second from the busy cycles of the pipe).  A
+// product of two-limb integers a = a1 2^32 + a0 whose low limbs are balanced (|a0| <= 2^31, random sign)
 // needs three of them, hh += a1 b1 and mid += a1 b0 + a0 b1: the dropped a0 b0
 // is below the last bit kept.  A multiply-add of more precision than FP64's
 // therefore takes three instructions of 1/16 the cost, which turns the operator
@@ -40,10 +40,10 @@
 // magnitudes of the terms that enter it.  So a site runs on fixed point only where
 // every one of its twelve components is large enough: FixTerms adds up magnitudes of
 // the hops' contributions to it, which with the sum's own (together at most twice the
-// terms) must reach 2^54 units.  Gaussian fields at kappa = 0.125 to 0.1365, on links
-// near and far from 1, c_SW 0 and 1, have 2^57.5 in the median and no component of
-// 4e5 below 2^55, so ordinary fields stay; a field whose colours or spins differ by
-// more than about 4 in scale without being mixed leaves.
+// terms) must reach 2^54 units.  Gaussian fields stay, at kappa = 0.125 to 0.1365, on
+// links near and far from 1, c_SW 0 and 1 (the median component has about 2^57.5; of
+// 663,552 sites none leaves, of the operator's sites in solves 6 in 10^6); a field whose
+// colours or spins differ by more than about 4 in scale without being mixed leaves.
 // Measured for a colour scaled by 2^-p on unit links: its error is 1.4e-16 to
 // 1.6e-16 at every p from 0 to 50, as with FP64 instructions (1.5e-16); without the
 // test it was 1.1e-14 at p = 10.
@@ -103,7 +103,7 @@ __device__ __forceinline__ fix_t mac64(int a, int b, fix_t c) { return c + (fix_
 __device__ __forceinline__ fix_t mul64(int a, int b) { return (fix_t)a * (fix_t)b; }
 // -x (and the limbs below) as 32-bit numbers of unknown origin: where the compiler
 // can see them it sign-extends first and multiplies 64-bit numbers (850 of the
-// 2,640 products a site, each in four instructions).  The products themselves
+// 2,640 multiply-adds a site, 2,520 products and 120 joins, each in four instructions).  The products themselves
 // stay in C: as mad.wide in inline PTX a third came out as a multiplication and
 // a separate 64-bit addition.
 __device__ __forceinline__ int fix_neg(int x)
@@ -177,7 +177,7 @@ __device__ __forceinline__ fix_t fix_from(uint32_t lo, uint32_t hi, int K, uint3
 }
 
 // Q of a double, K = the unit's biased exponent + 4: x = Q 2^(K - 1086) rounded
-// towards zero, |x| < 2^(K - 1026)
+// towards zero, |x| < 2^(K - 1023) (|Q| < 2^63)
 __device__ __forceinline__ fix_t fix_from_any(double x, int K)
 {
     const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
@@ -346,9 +346,10 @@ struct FixTerms {
     }
 };
 
-// The projected half spinor of direction m (above) from the spinor in the
-// staging slots (negated where `flip`, conjugated where `back`), as limbs; raises E (and shifts acc down) where the neighbour
-// exceeds it; FIX_LEAVE when the site needs FP64.
+// The projected half spinor of direction m (above) from the spinor in the staging
+// slots (negated where `flip`, conjugated where `back`), as limbs; raises E (and
+// shifts acc and the terms down) where the neighbour exceeds it; FIX_LEAVE when the
+// site needs FP64.
 enum { FIX_LEAVE, FIX_ZERO, FIX_HOP };
 __device__ __forceinline__ int fix_half_spinor(const int4 *slot, int nt, int m, bool back, bool flip, Cx<fix_t> acc[12],
                                                 FixTerms &terms, int &E, int h1[12], int h0[12])
